@@ -10,6 +10,15 @@ namespace rlbmk {
 // MODE_STEP_LATTICE: a step of the on-lattice rule (perfect streaming by the
 // integer stencil vector of each population, no interpolation).
 // MODE_Q (a bit added to STEP, INIT, MOMENTS): the quantum statistics.
+// How the two sites of a lane of the quadrant kernel lie (rlbm_quad.cuh).
+//   kMapRow     x, x + 1 of one row (nx even): 64 x 1 tiles, 8-byte (4-byte) centre loads
+//   kMapCol     x of rows y, y + 1 (ny > 1, any nx): 32 x 2 tiles; a population needs three
+//               rows for two sites, and the interpolation along x of the middle row serves
+//               both sites: three interpolations along x instead of four, 1.5 instead of 2
+//               reads of a population from the L2
+//   kMapSplit   x, x + 32 of one row (ny = 1, any nx): 64 x 1 tiles
+enum QuadMap { kMapRow = 0, kMapCol = 1, kMapSplit = 2 };
+
 enum Mode { MODE_STEP = 0, MODE_INIT = 1, MODE_MOMENTS = 2, MODE_STEP_LATTICE = 3, MODE_Q = 4 };
 
 constexpr int kMaxN = 5;
@@ -55,6 +64,15 @@ struct KernelArgs {
     double *out[6];                            // MODE_MOMENTS fields
     const unsigned long long *masks; // per warp: bit k = (v_x >= 0), (v_y >= 0) of its population k (k < 64)
     const void *pairtab; // npop x 3 float4: paired constants of the two-sites-per-lane kernel (FP32 arithmetic)
+    const void *quadtab; // N+1 shells x K/4 quads x 3 float4: (c,c,s,s), (cos 2t, cos 2t, sin 2t, sin 2t), third harmonic
+                         // (FP64 storage: c, s, cos 2t, sin 2t, cos 3t, sin 3t)
+    // quadrant kernels (N <= 3), in the parameter space so that no load waits for them:
+    // (N+1)^3 projection weights times the shell's population weight (stored units) and the
+    // shell folds alpha_r p_r, alpha_r p_r^2, as double-floats (hi, lo)
+    float2 rq[64], shellq[8];
+    double rqd[64];      // the projection weights in FP64 (FP64 storage)
+    float beta_f;        // stored-unit offset (FP32)
+    int cluster;         // CTAs per cluster of the many-angle quadrant kernel
     const int2 *shifts;  // npop: integer stencil vectors of the on-lattice rule (else NULL)
     double *qeta;        // quantum statistics: per site, eta = ln z of the last solve (the next
                          // step's Newton start; NaN: none yet), else NULL
@@ -127,6 +145,17 @@ __host__ __device__ constexpr size_t pair_smem_total(int N, int G, bool bulk, in
 {
     return pair_smem_bytes(N, G, bulk, elem_bytes, two_d) +
            (elem_bytes == 4 && pair_split(N, G) ? size_t(split_rows(N)) * kPairSites * 4 : 0);
+}
+
+// Many-angle quadrant kernel (rlbm_quad_cluster_kernel): CTAs per cluster, two per shell
+// (6 or 8, the portable size), warps per CTA, and dynamic shared memory: the angular sums of
+// the cluster's CTAs and of this CTA's warps, the per-site rows, 1 KB per quad.
+__host__ __device__ constexpr int quad_cluster_size(int N) { return 2 * (N + 1); }
+constexpr int kQuadClusterWarps = 10;
+__host__ __device__ constexpr size_t quad_cluster_smem(int N, int K)
+{
+    return size_t(5 * quad_cluster_size(N) + 5 * kQuadClusterWarps + pair_site_rows(N)) * kPairSites * 4 +
+           size_t((K / 4 + 1) / 2) * 1024;
 }
 
 // Arguments of the persistent TMA-staged step kernel.
@@ -207,35 +236,53 @@ cudaError_t launch_f16_n45(int mode, int N, int P, bool two_d, bool full, dim3 g
                            size_t smem, cudaStream_t st, const KernelArgs &a);
 cudaError_t launch_bf16_n45(int mode, int N, int P, bool two_d, bool full, dim3 grid, dim3 block,
                             size_t smem, cudaStream_t st, const KernelArgs &a);
-// Two-sites-per-lane step kernel (rlbm_pair.cuh): 64-site tiles, PP in {8, 12, 16, 24, 32};
-// bulk: interior tiles staged through shared memory by cp.async.bulk.
-// Two-sites-per-lane kernels: one compile unit per storage, order N and form
-// (p plain, b bulk-staged first pass), compiled in parallel; the dispatchers
-// below pick the unit.
+// Bulk-staged two-sites-per-lane step kernel (rlbm_pair.cuh): 64-site tiles, PP in
+// {8, 12, 16, 24, 32}; one compile unit per storage and order N, compiled in parallel.
 #define RLBM_DECLARE_PAIR(name)                                                                          \
-    cudaError_t launch_pair_##name##_n2p(int PP, bool two_d, dim3 grid, dim3 block, size_t smem,         \
-                                         cudaStream_t st, const KernelArgs &a);                          \
     cudaError_t launch_pair_##name##_n2b(int PP, bool two_d, dim3 grid, dim3 block, size_t smem,         \
-                                         cudaStream_t st, const KernelArgs &a);                          \
-    cudaError_t launch_pair_##name##_n3p(int PP, bool two_d, dim3 grid, dim3 block, size_t smem,         \
                                          cudaStream_t st, const KernelArgs &a);                          \
     cudaError_t launch_pair_##name##_n3b(int PP, bool two_d, dim3 grid, dim3 block, size_t smem,         \
                                          cudaStream_t st, const KernelArgs &a);                          \
-    inline cudaError_t launch_pair_##name(int N, int PP, bool two_d, bool bulk, dim3 grid, dim3 block,   \
-                                          size_t smem, cudaStream_t st, const KernelArgs &a)             \
+    inline cudaError_t launch_pair_##name(int N, int PP, bool two_d, dim3 grid, dim3 block, size_t smem, \
+                                          cudaStream_t st, const KernelArgs &a)                          \
     {                                                                                                    \
-        if (N == 2)                                                                                      \
-            return bulk ? launch_pair_##name##_n2b(PP, two_d, grid, block, smem, st, a)                  \
-                        : launch_pair_##name##_n2p(PP, two_d, grid, block, smem, st, a);                 \
-        if (N == 3)                                                                                      \
-            return bulk ? launch_pair_##name##_n3b(PP, two_d, grid, block, smem, st, a)                  \
-                        : launch_pair_##name##_n3p(PP, two_d, grid, block, smem, st, a);                 \
+        if (N == 2) return launch_pair_##name##_n2b(PP, two_d, grid, block, smem, st, a);                \
+        if (N == 3) return launch_pair_##name##_n3b(PP, two_d, grid, block, smem, st, a);                \
         return cudaErrorInvalidValue;                                                                    \
     }
 RLBM_DECLARE_PAIR(f32)
 RLBM_DECLARE_PAIR(f16)
 RLBM_DECLARE_PAIR(bf16)
 #undef RLBM_DECLARE_PAIR
+// Quadrant step kernel (rlbm_quad.cuh); map: QuadMap, how a lane's two sites lie.
+#define RLBM_DECLARE_QUAD(name)                                                                          \
+    cudaError_t launch_quad_##name##_n2(int PP, int map, bool two_d, dim3 block, size_t smem,            \
+                                        cudaStream_t st, const KernelArgs &a);                           \
+    cudaError_t launch_quad_##name##_n3(int PP, int map, bool two_d, dim3 block, size_t smem,            \
+                                        cudaStream_t st, const KernelArgs &a);                           \
+    inline cudaError_t launch_quad_##name(int N, int PP, int map, bool two_d, dim3 block, size_t smem,   \
+                                          cudaStream_t st, const KernelArgs &a)                          \
+    {                                                                                                    \
+        if (N == 2) return launch_quad_##name##_n2(PP, map, two_d, block, smem, st, a);                  \
+        if (N == 3) return launch_quad_##name##_n3(PP, map, two_d, block, smem, st, a);                  \
+        return cudaErrorInvalidValue;                                                                    \
+    }
+RLBM_DECLARE_QUAD(f32)
+RLBM_DECLARE_QUAD(stat_f32) // the quantum statistics
+RLBM_DECLARE_QUAD(f16)
+RLBM_DECLARE_QUAD(bf16)
+#undef RLBM_DECLARE_QUAD
+cudaError_t launch_quad_f64_n2(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
+cudaError_t launch_quad_f64_n3(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
+// many angles (FP32 storage): clusters of CTAs
+cudaError_t launch_quad_cluster_f32_n2(int map, bool two_d, cudaStream_t st, const KernelArgs &a);
+cudaError_t launch_quad_cluster_f32_n3(int map, bool two_d, cudaStream_t st, const KernelArgs &a);
+inline cudaError_t launch_quad_cluster_f32(int N, int map, bool two_d, cudaStream_t st, const KernelArgs &a)
+{
+    if (N == 2) return launch_quad_cluster_f32_n2(map, two_d, st, a);
+    if (N == 3) return launch_quad_cluster_f32_n3(map, two_d, st, a);
+    return cudaErrorInvalidValue;
+}
 // several population groups per warp (FP32 storage)
 cudaError_t launch_pair_groups_f32_n2(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                       const KernelArgs &a);
@@ -249,11 +296,19 @@ inline cudaError_t launch_pair_groups_f32(int N, int PP, bool two_d, dim3 grid, 
     return cudaErrorInvalidValue;
 }
 
+// Offsets of PairTmaSmem, formed once on the host (the kernel's warps would each repeat
+// about 60 integer instructions).
+struct PairTmaLayout {
+    unsigned stage, tab, red, sres, bar;
+    int alias;
+};
+
 // Arguments of the tile-staged two-sites-per-lane kernel (rlbm_pair_tma.cuh).
 struct alignas(128) PairTmaArgs {
     CUtensorMap cmap; // 3D map over the input buffer {nx, ny, npop}, box {BW, 1, CB}: centre rows
     CUtensorMap pmap; // the same map with box {BW, 1, DB}: pull rows
     KernelArgs a;
+    PairTmaLayout layout;
     int CB, ncbox;    // populations per centre box, boxes per tile (CB ncbox = npop)
     int DB, npbox;    // populations per pull-row chunk, chunks per tile (DB npbox = npop)
     unsigned long long chunk_up[4]; // bit c: chunk c pulls from row y - 1 (its v_y >= 0), else y + 1
@@ -310,6 +365,11 @@ RLBM_DECLARE_PAIR_TMA(f32)
 RLBM_DECLARE_PAIR_TMA(f16)
 RLBM_DECLARE_PAIR_TMA(bf16)
 #undef RLBM_DECLARE_PAIR_TMA
+
+// Free streaming of thin grids (rlbm_free.cu): nsteps <= kFreeSteps steps of every
+// population in one launch, ny <= kFreeRows, FP64 or FP32 storage.
+constexpr int kFreeSteps = 32, kFreeRows = 4;
+cudaError_t launch_free(bool fp64, int N, int npop, int nsteps, cudaStream_t st, const KernelArgs &a);
 
 // Batched persistent form (rlbm_batch.cuh).
 constexpr int kBatchWarps = 6;

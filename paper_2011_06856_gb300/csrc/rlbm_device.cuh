@@ -299,7 +299,11 @@ __device__ __forceinline__ bool landau_fast(const LR *m, LR &n, LR &eps, LR &U0,
     const LR b0 = r_div(LR(4) * M, LR(3) * E + r_sqrt(disc > LR(0) ? disc : LR(0)));
     LR lam = E - b0 * M;
     if ((lam * lam + c1) * lam - c0 < LR(0)) lam = E;
-    const LR tol = LR(sizeof(LR) == 8 ? 4e-16 : 2e-7);
+    // Newton converges quadratically: after a last step of tol lam the error is about
+    // tol^2 (3 lam^2 / P'(lam)), below the rounding of P itself.  A tolerance near the
+    // rounding unit would be missed by noise and run the loop to its bound (the FP32 solve
+    // of a tile took 2.5 times as long).
+    const LR tol = LR(sizeof(LR) == 8 ? 2e-9 : 5e-5);
 #pragma unroll 1
     for (int it = 0; it < 24; ++it) {
         const LR P = (lam * lam + c1) * lam - c0;

@@ -182,5 +182,17 @@ __device__ __forceinline__ df2 scale(df2 x, float b)
     return p_fast_two_sum(p, pfma(x.lo, bb, pfma(x.hi, bb, pneg(p))));
 }
 __device__ __forceinline__ float2 to_float2(df2 x) { return padd(x.hi, x.lo); }
+__device__ __forceinline__ df2 operator*(df2 x, df2 y)
+{
+    const float2 p = pmul(x.hi, y.hi);
+    const float2 e = pfma(x.hi, y.lo, pfma(x.lo, y.hi, pfma(x.hi, y.hi, pneg(p))));
+    return p_fast_two_sum(p, e);
+}
+__device__ __forceinline__ df2 operator*(df2 x, float b) { return scale(x, b); }
+__device__ __forceinline__ df2 operator+(df2 x, float b)
+{
+    const df2 s = p_two_sum(x.hi, make_float2(b, b));
+    return p_fast_two_sum(s.hi, padd(s.lo, x.lo));
+}
 
 } // namespace rlbmk

@@ -507,7 +507,25 @@ rlbm_status build_tables(rlbm_t *h)
     std::vector<int> shifts;
     if (q.onlat)
         for (int i = 0; i < npop; ++i) { shifts.push_back(q.sx[i]); shifts.push_back(q.sy[i]); }
-    const size_t o_shift = o_pair + align256(ptab.size() * 4);
+    // quadrant tables (N <= 3, K a multiple of 4): the harmonics of the
+    // base angle of each quadruple, and the projection weights with the shell's weight
+    std::vector<double> qtab, rq;
+    if (N <= 3 && K % 4 == 0 && !q.onlat) {
+        for (int r = 0; r <= N; ++r)
+            for (int j = 0; j < K / 4; ++j) {
+                const int i = r * K + j;
+                const double th = (j + r / double(N + 1)) * (2.0 * kPi / K);
+                const double c = q.vx[i], s = q.vy[i];
+                const double v[6] = {c, s, std::cos(2 * th), std::sin(2 * th), std::cos(3 * th), std::sin(3 * th)};
+                for (double e : v) // FP32 arithmetic: each twice, for the packed operations
+                    qtab.insert(qtab.end(), r64 ? 1 : 2, e);
+            }
+        rq = rt;
+        for (int r = 0; r <= N; ++r)
+            for (int t = 0; t < (N + 1) * (N + 1); ++t) rq[size_t(r) * (N + 1) * (N + 1) + t] *= pop[size_t(r) * K * TW + 4];
+    }
+    const size_t o_quad = o_pair + align256(ptab.size() * 4);
+    const size_t o_shift = o_quad + align256(qtab.size() * rs);
     const size_t total = o_shift + align256(shifts.size() * sizeof(int));
     std::vector<unsigned char> blob(total, 0);
     if (r64) put<double>(blob, o_pop, pop); else put<float>(blob, o_pop, pop);
@@ -515,6 +533,7 @@ rlbm_status build_tables(rlbm_t *h)
     else { put<float>(blob, o_shell, shell); put<float>(blob, o_rt, rt); }
     std::memcpy(blob.data() + o_mask, masks.data(), masks.size() * sizeof(unsigned long long));
     put<float>(blob, o_pair, ptab);
+    if (r64) put<double>(blob, o_quad, qtab); else put<float>(blob, o_quad, qtab);
     std::memcpy(blob.data() + o_shell2, shell2.data(), shell2.size() * 4);
     std::memcpy(blob.data() + o_rt2, rt2.data(), rt2.size() * 4);
     if (!shifts.empty()) std::memcpy(blob.data() + o_shift, shifts.data(), shifts.size() * sizeof(int));
@@ -573,6 +592,14 @@ rlbm_status build_tables(rlbm_t *h)
     a.rtab2 = reinterpret_cast<const float2 *>((const unsigned char *)h->d_tabs + o_rt2);
     a.masks = reinterpret_cast<const unsigned long long *>((const unsigned char *)h->d_tabs + o_mask);
     a.pairtab = ptab.empty() ? nullptr : (const unsigned char *)h->d_tabs + o_pair;
+    a.quadtab = qtab.empty() ? nullptr : (const unsigned char *)h->d_tabs + o_quad;
+    if (!qtab.empty()) {
+        const std::vector<float> rq2 = split(rq);
+        std::memcpy(a.rq, rq2.data(), rq2.size() * 4);
+        std::memcpy(a.shellq, shell2.data(), shell2.size() * 4);
+        std::memcpy(a.rqd, rq.data(), rq.size() * 8);
+    }
+    a.beta_f = float(beta);
     a.shifts = shifts.empty() ? nullptr : reinterpret_cast<const int2 *>((const unsigned char *)h->d_tabs + o_shift);
     a.status = h->d_status;
     a.ctr = reinterpret_cast<unsigned *>(h->d_status + 1);
@@ -654,13 +681,42 @@ bool pair_bulk_possible(const rlbm_t *h)
     return (size_t(h->grid.nx) * storage_size(h->prec)) % 16 == 0 && reinterpret_cast<uintptr_t>(h->buf) % 16 == 0;
 }
 
+// The quadrant kernel (rlbm_quad.cuh): FP32 per-population arithmetic, a collision,
+// N <= 3, K a multiple of P (so of 4), one population group.  With nx even it is the two-sites-per-lane
+// kernel (kind 2); for any nx it also takes the place of the per-tile kernel (kind 0),
+// with a lane's sites in two rows (ny > 1) or 32 apart (ny = 1).
+bool quad_possible(const rlbm_t *h, int P)
+{
+    int gs = 0, ng = 0;
+    return h->prec != RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && !h->stat &&
+           (P == 8 || P == 12 || P == 16 || P == 24 || P == 32) && h->K % P == 0 &&
+           group_tiling(h->N, h->K, P, gs, ng) && ng == 1;
+}
+
+cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
+{
+    const dim3 block(32, h->Gs, h->N + 1);
+    const bool two_d = h->grid.ny > 1;
+    const size_t smem = rlbmk::pair_smem_bytes(h->N, h->G, false, int(storage_size(h->prec)), two_d);
+    cudaError_t e;
+    switch (h->prec) {
+    case RLBM_FP32: e = rlbmk::launch_quad_f32(h->N, h->P, map, two_d, block, smem, h->stream, a); break;
+    case RLBM_FP16_DEV:
+    case RLBM_FP16_NORM: e = rlbmk::launch_quad_f16(h->N, h->P, map, two_d, block, smem, h->stream, a); break;
+    default: e = rlbmk::launch_quad_bf16(h->N, h->P, map, two_d, block, smem, h->stream, a); break;
+    }
+    if (e == cudaSuccess) ++h->launches;
+    return e;
+}
+
 cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
+    if (!h->pair_bulk && h->R == 1) return launch_quad(h, rlbmk::kMapRow, a);
     const dim3 grid((h->grid.nx + rlbmk::kPairSites - 1) / rlbmk::kPairSites, h->grid.ny);
     const dim3 block(32, h->G);
     // the population-groups kernel has no bulk staging
-    const bool two_d = h->grid.ny > 1, bulk = h->pair_bulk && h->R == 1;
-    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, bulk, int(storage_size(h->prec)), two_d);
+    const bool two_d = h->grid.ny > 1;
+    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, h->R == 1, int(storage_size(h->prec)), two_d);
     cudaError_t e;
     if (h->R > 1) { // several population groups per warp (FP32 storage: pair_possible)
         e = rlbmk::launch_pair_groups_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a);
@@ -668,12 +724,12 @@ cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
         return e;
     }
     switch (h->prec) {
-    case RLBM_FP32: e = rlbmk::launch_pair_f32(h->N, h->P, two_d, bulk, grid, block, smem, h->stream, a); break;
+    case RLBM_FP32: e = rlbmk::launch_pair_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a); break;
     case RLBM_FP16_DEV:
     case RLBM_FP16_NORM:
-        e = rlbmk::launch_pair_f16(h->N, h->P, two_d, bulk, grid, block, smem, h->stream, a);
+        e = rlbmk::launch_pair_f16(h->N, h->P, two_d, grid, block, smem, h->stream, a);
         break;
-    default: e = rlbmk::launch_pair_bf16(h->N, h->P, two_d, bulk, grid, block, smem, h->stream, a); break;
+    default: e = rlbmk::launch_pair_bf16(h->N, h->P, two_d, grid, block, smem, h->stream, a); break;
     }
     if (e == cudaSuccess) ++h->launches;
     return e;
@@ -682,7 +738,7 @@ cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
 // with bps set: only the occupancy query (CTAs per SM)
 cudaError_t launch_pair_tma_raw(rlbm_t *h, const rlbmk::PairTmaArgs &ta, int *bps)
 {
-    const dim3 block(32, h->G);
+    const dim3 block(32, h->Gs, h->N + 1);
     const bool two_d = h->grid.ny > 1;
     switch (h->prec) {
     case RLBM_FP32: return rlbmk::launch_pair_tma_f32(h->N, h->P, two_d, block, h->ptma_smem, h->stream, ta, bps);
@@ -745,6 +801,8 @@ cudaError_t launch_step(rlbm_t *h, int from)
         h->stall_next = false;
         return launch_pair(h, a);
     }
+    const int map = h->grid.ny > 1 ? rlbmk::kMapCol : rlbmk::kMapSplit; // for any nx
+    if (quad_possible(h, h->P)) return launch_quad(h, map, a);
     return launch(h, rlbmk::MODE_STEP, a);
 }
 
@@ -886,7 +944,8 @@ rlbm_status setup_pair_tma(rlbm_t *h)
     RLBM_CUDA(h, cudaGetDevice(&dev));
     RLBM_CUDA(h, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     RLBM_CUDA(h, cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
-    const size_t need = rlbmk::PairTmaSmem(h->N, h->G, npop, int(es), two_d).total;
+    const rlbmk::PairTmaSmem L(h->N, h->G, npop, int(es), two_d);
+    const size_t need = L.total;
     if (need > size_t(max_smem)) return RLBM_OK;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -921,6 +980,7 @@ rlbm_status setup_pair_tma(rlbm_t *h)
             }
         }
         ta.a = h->base;
+        ta.layout = {unsigned(L.stage), unsigned(L.tab), unsigned(L.red), unsigned(L.sres), unsigned(L.bar), L.alias ? 1 : 0};
         ta.CB = CB;
         ta.ncbox = ncbox;
         ta.DB = DB;
@@ -1709,13 +1769,17 @@ rlbm_status batch_check(rlbm_batch *b)
 
 constexpr int kBatchStreams = 16;
 
+// Step kernel of a problem in the stream pool at tiling P: two sites per lane, in one
+// row for an even nx, else (kind 0) in the quadrant kernel's forms for any nx.
+int solo_kind_for(const rlbm_t *h, int P) { return pair_possible(h, P) ? 2 : 0; }
+
 // Smallest two-sites-per-lane tiling of a problem (more, lighter warps per
 // SM), else the per-tile kernel with the default tiling.
 void solo_default(const rlbm_t *h, int &P, int &kind)
 {
     static const int sizes[] = {8, 12, 16, 24, 32};
     for (int v : sizes)
-        if (pair_possible(h, v)) { P = v; kind = pair_bulk_possible(h) ? 3 : 2; return; }
+        if (pair_possible(h, v) || quad_possible(h, v)) { P = v; kind = solo_kind_for(h, v); return; }
     int gs = 0, ng = 0;
     choose_tiling(h->N, h->K, P, gs, ng);
     kind = 0;
@@ -2072,7 +2136,7 @@ rlbm_status rlbm_batch_autotune(rlbm_batch_t *b, int steps_per_trial, float *bes
         for (int P : psizes) {
             std::vector<int> members;
             for (int i : c.second)
-                if (pair_possible(b->probs[i], P) && !(b->solo_kind[i] >= 2 && b->solo_P[i] == P)) members.push_back(i);
+                if ((pair_possible(b->probs[i], P) || quad_possible(b->probs[i], P)) && b->solo_P[i] != P) members.push_back(i);
             if (members.empty()) continue;
             std::vector<int> oldP, oldK;
             if (!st) st = batch_sync_all(b);
@@ -2080,7 +2144,7 @@ rlbm_status rlbm_batch_autotune(rlbm_batch_t *b, int steps_per_trial, float *bes
                 oldP.push_back(b->solo_P[i]);
                 oldK.push_back(b->solo_kind[i]);
                 b->solo_P[i] = P;
-                b->solo_kind[i] = pair_bulk_possible(b->probs[i]) ? 3 : 2;
+                b->solo_kind[i] = solo_kind_for(b->probs[i], P);
                 if (!st) st = retile(b->probs[i], P, b->solo_kind[i]);
             }
             float ms = 0.f;

@@ -81,11 +81,24 @@ __device__ __forceinline__ bool pbar_wait(unsigned bar, unsigned parity, long lo
     return true;
 }
 
+// f16 -> f32 by the mixed-precision addition of -0 (exact; one cycle of the FMA pipe, the
+// conversion instruction takes two)
+__device__ __forceinline__ float half_bits_to_float(unsigned short u)
+{
+    float v;
+    asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(v) : "h"(u), "f"(-0.f));
+    return v;
+}
+__device__ __forceinline__ float2 half2_bits_to_float2(unsigned u)
+{
+    return make_float2(half_bits_to_float((unsigned short)u), half_bits_to_float((unsigned short)(u >> 16)));
+}
+
 template <class St> __device__ __forceinline__ float2 lds2(const St *p);
 template <> __device__ __forceinline__ float2 lds2<float>(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 template <> __device__ __forceinline__ float2 lds2<__half>(const __half *p)
 {
-    return __half22float2(*reinterpret_cast<const __half2 *>(p));
+    return half2_bits_to_float2(*reinterpret_cast<const unsigned *>(p));
 }
 template <> __device__ __forceinline__ float2 lds2<__nv_bfloat16>(const __nv_bfloat16 *p)
 {
@@ -94,7 +107,10 @@ template <> __device__ __forceinline__ float2 lds2<__nv_bfloat16>(const __nv_bfl
 }
 template <class St> __device__ __forceinline__ float lds1(const St *p);
 template <> __device__ __forceinline__ float lds1<float>(const float *p) { return *p; }
-template <> __device__ __forceinline__ float lds1<__half>(const __half *p) { return __half2float(*p); }
+template <> __device__ __forceinline__ float lds1<__half>(const __half *p)
+{
+    return half_bits_to_float(*reinterpret_cast<const unsigned short *>(p));
+}
 template <> __device__ __forceinline__ float lds1<__nv_bfloat16>(const __nv_bfloat16 *p)
 {
     return __bfloat162float(*p);
@@ -125,15 +141,13 @@ template <> struct PIo<__half> {
     {
         unsigned u;
         asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(u) : "l"(p));
-        __half2 h;
-        memcpy(&h, &u, 4);
-        return __half22float2(h);
+        return half2_bits_to_float2(u);
     }
     static __device__ __forceinline__ float ld1(const __half *p)
     {
         unsigned short u;
         asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(u) : "l"(p));
-        return __half2float(__ushort_as_half(u));
+        return half_bits_to_float(u);
     }
     static __device__ __forceinline__ void st2(__half *p, float2 v, unsigned &rng)
     {
@@ -391,7 +405,7 @@ __device__ __forceinline__ void pair_shell_coefficients(const KernelArgs &a, int
 // multiple of PP); TWO_D: ny > 1; BULK: staged pass 1 on interior tiles (row
 // pitch a multiple of 16 bytes, buffers 16-byte aligned).  Requires nx even
 // (paired access) and a collision (tau finite).
-template <class St, int N, int PP, bool TWO_D, bool BULK>
+template <class St, int N, int PP, bool TWO_D>
 __global__ void __launch_bounds__(kMaxWarps * 32, PP <= 16 ? 2 : 1) rlbm_pair_kernel(const KernelArgs a)
 {
     constexpr int NC = 2 * N + 1;
@@ -448,7 +462,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, PP <= 16 ? 2 : 1) rlbm_pair_ke
     constexpr int BW = kPairSites + 2 * HX;      // staged row width (elements)
     constexpr int RW = TWO_D ? 2 : 1;            // staged rows per population
     constexpr int NCH = PP / kPairChunk;         // chunks per warp
-    const bool staged = BULK && x0 >= HX && x0 + kPairSites + HX <= a.nx;
+    const bool staged = x0 >= HX && x0 + kPairSites + HX <= a.nx;
     bool good = true; // every bounded wait of this warp completed
     if (staged) {
         static_assert(PP % kPairChunk == 0, "chunking");
@@ -546,7 +560,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, PP <= 16 ? 2 : 1) rlbm_pair_ke
     __syncthreads();
     constexpr bool DD = sizeof(St) == 4; // FP32 storage: FP64-class per-site part
     if (DD && pair_split(N, G)) { // double-float, split over the warps by sample direction
-        float *fr = reinterpret_cast<float *>(smem_raw + pair_smem_bytes(N, G, BULK, 4, TWO_D));
+        float *fr = reinterpret_cast<float *>(smem_raw + pair_smem_bytes(N, G, true, 4, TWO_D));
         const int tid = g * 32 + lane;
         site_split_dd<N, kPairSites>(a, red, G, tid, G * 32, x0 + tid < a.nx, sres, fr,
                                      fr + kSplitFrameRows(N) * kPairSites);
@@ -779,14 +793,13 @@ static cudaError_t launch_pair_groups_n(int PP, bool two_d, dim3 grid, dim3 bloc
     }
 }
 
-// The two-sites-per-lane kernel of storage St, order N, plain (BULK false) or
-// bulk-staged first pass: the instances of one compile unit.
-template <class St, int N, int PP, bool BULK>
+// The bulk-staged two-sites-per-lane kernel of storage St, order N: the instances of one
+// compile unit.
+template <class St, int N, int PP>
 static cudaError_t launch_pair_one(bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                    const KernelArgs &a)
 {
-    void (*k)(const KernelArgs) =
-        two_d ? rlbm_pair_kernel<St, N, PP, true, BULK> : rlbm_pair_kernel<St, N, PP, false, BULK>;
+    void (*k)(const KernelArgs) = two_d ? rlbm_pair_kernel<St, N, PP, true> : rlbm_pair_kernel<St, N, PP, false>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -795,16 +808,16 @@ static cudaError_t launch_pair_one(bool two_d, dim3 grid, dim3 block, size_t sme
     return cudaGetLastError();
 }
 
-template <class St, int N, bool BULK>
+template <class St, int N>
 static cudaError_t launch_pair_nb(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                   const KernelArgs &a)
 {
     switch (PP) {
-    case 8: return launch_pair_one<St, N, 8, BULK>(two_d, grid, block, smem, st, a);
-    case 12: return launch_pair_one<St, N, 12, BULK>(two_d, grid, block, smem, st, a);
-    case 16: return launch_pair_one<St, N, 16, BULK>(two_d, grid, block, smem, st, a);
-    case 24: return launch_pair_one<St, N, 24, BULK>(two_d, grid, block, smem, st, a);
-    case 32: return launch_pair_one<St, N, 32, BULK>(two_d, grid, block, smem, st, a);
+    case 8: return launch_pair_one<St, N, 8>(two_d, grid, block, smem, st, a);
+    case 12: return launch_pair_one<St, N, 12>(two_d, grid, block, smem, st, a);
+    case 16: return launch_pair_one<St, N, 16>(two_d, grid, block, smem, st, a);
+    case 24: return launch_pair_one<St, N, 24>(two_d, grid, block, smem, st, a);
+    case 32: return launch_pair_one<St, N, 32>(two_d, grid, block, smem, st, a);
     default: return cudaErrorInvalidValue;
     }
 }

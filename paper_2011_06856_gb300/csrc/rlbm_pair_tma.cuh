@@ -33,7 +33,7 @@
 // waits (again bounded) for its copies and returns without storing.
 #pragma once
 
-#include "rlbm_pair.cuh"
+#include "rlbm_quad.cuh"
 #include "rlbm_tma.cuh"
 
 namespace rlbmk {
@@ -43,37 +43,22 @@ template <class St> struct PairTmaGeom {
     static constexpr int BW = kPairSites + 2 * HX;  // box width in x (a multiple of 16 bytes)
 };
 
-// 16-bit pair stores with the stochastic-rounding conversion (the first
-// source operand lands in the upper half: the site at the higher address)
-template <class St> __device__ __forceinline__ void st2_rs(St *p, float2 v, unsigned rbits);
-template <> __device__ __forceinline__ void st2_rs<__half>(__half *p, float2 v, unsigned rbits)
-{
-    unsigned d;
-    asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.y), "f"(v.x), "r"(rbits));
-    *reinterpret_cast<unsigned *>(p) = d;
-}
-template <> __device__ __forceinline__ void st2_rs<__nv_bfloat16>(__nv_bfloat16 *p, float2 v, unsigned rbits)
-{
-    unsigned d;
-    asm("cvt.rs.satfinite.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.y), "f"(v.x), "r"(rbits));
-    *reinterpret_cast<unsigned *>(p) = d;
-}
-
 template <class St, int N, int PP, bool TWO_D>
 __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
 {
     constexpr int NC = 2 * N + 1;
-    constexpr int PQ = 3; // float4 per population in the pair table
+    constexpr int QW = PP / 4; // quads per warp
     constexpr int HX = PairTmaGeom<St>::HX, BW = PairTmaGeom<St>::BW;
     constexpr int RW = TWO_D ? 2 : 1;
     const KernelArgs &a = ta.a;
     extern __shared__ __align__(16) unsigned char smem_pt[];
     // TMA destinations: align the base to 1 KB (the host adds the slack)
     unsigned char *sm = smem_pt + ((1024u - (smem_u32(smem_pt) & 1023u)) & 1023u);
-    const int lane = threadIdx.x, g = threadIdx.y, G = blockDim.y;
+    const PairTmaLayout &L = ta.layout;
+    const int lane = threadIdx.x, q = threadIdx.y, Gs = blockDim.y, r = threadIdx.z;
+    const int g = r * Gs + q, G = Gs * (N + 1);
     const int tid = g * 32 + lane, nthr = G * 32;
     const int npop = a.K * (N + 1);
-    const PairTmaSmem L(N, G, npop, int(sizeof(St)), TWO_D);
     St *stage = reinterpret_cast<St *>(sm + L.stage); // [RW][npop][BW]
     float4 *tab = reinterpret_cast<float4 *>(sm + L.tab);
     float *red = reinterpret_cast<float *>(sm + L.red);   // [5][G][64]
@@ -83,6 +68,7 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
     const int ym = TWO_D ? bc_index(y - 1, a.ny, a.bcy) : y;
     const int yp = TWO_D ? bc_index(y + 1, a.ny, a.bcy) : y;
 
+    const unsigned seed = __ldcg(a.ctr); // early: its latency passes behind the copies
     if (tid == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
@@ -103,10 +89,10 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
             }
         }
     }
-    // while the copies fly: the pair table into shared memory
+    // while the copies fly: the quad table into shared memory
     {
-        const float4 *gt = reinterpret_cast<const float4 *>(a.pairtab);
-        for (int e = tid; e < npop * PQ; e += nthr) tab[e] = __ldg(gt + e);
+        const float4 *gt = reinterpret_cast<const float4 *>(a.quadtab);
+        for (int e = tid; e < (npop >> 2) * 3; e += nthr) tab[e] = __ldg(gt + e);
     }
     const bool arrived = mbar_wait_bounded(bar, 0, a.wait_cycles);
     if (__syncthreads_or(!arrived)) {
@@ -140,88 +126,65 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
 
     const int xl = x0 + 2 * lane;
     const bool act = xl < a.nx;
-    const int r = g / a.Gs, q = g % a.Gs;
-    const int i0 = r * a.K + q * PP;
-    const St *cb = stage + size_t(i0) * BW + HX + 2 * lane;         // centre row, this lane's pair
-    const St *pb = stage + size_t(npop + i0) * BW + HX + 2 * lane;  // pull row
-    const float4 *tb = tab + size_t(i0) * PQ;
-    const unsigned long long mx = __ldg(a.masks + 2 * g);
+    const int K4 = a.K >> 2, i0 = r * a.K + q * QW; // population a = 0 of the warp's first quad
+    const St *cb = stage + size_t(i0) * BW + HX + 2 * lane;        // centre row, this lane's pair
+    const St *pb = stage + size_t(npop + i0) * BW + HX + 2 * lane; // pull row
+    const int aw = K4 * BW;                                        // to the quad's next population
+    const float4 *tb = tab + size_t(r * K4 + q * QW) * 3;
 
-    // pass 1: bilinear pull from shared memory, five angular sums
+    // pass 1: bilinear pull from shared memory, harmonic sums
     float2 fs[PP];
-    float2 s0 = f2(0.f, 0.f), sc = f2(0.f, 0.f), ss = f2(0.f, 0.f), scc = f2(0.f, 0.f), scs = f2(0.f, 0.f);
+    QuadSums sums = quad_sums_zero();
 #pragma unroll
-    for (int k = 0; k < PP; ++k) {
-        const bool px = (mx >> k) & 1ull; // v_x >= 0: pull from x - 1
-        const St *ra = cb + k * BW;
-        const float2 C = lds2<St>(ra);
-        const float e = lds1<St>(ra + (px ? -1 : 2));
-        const float4 t0 = tb[k * PQ], t1 = tb[k * PQ + 1]; // (c,c,s,s), (|c|,|c|,|s|,|s|)
-        const float2 B = px ? f2(e, C.x) : f2(C.y, e);
-        const float2 ac = f2(t1.x, t1.y);
-        float2 v = __ffma2_rn(ac, f2sub(B, C), C);
-        if (TWO_D) {
-            const St *rb = pb + k * BW;
-            const float2 C2 = lds2<St>(rb);
-            const float e2 = lds1<St>(rb + (px ? -1 : 2));
-            const float2 B2 = px ? f2(e2, C2.x) : f2(C2.y, e2);
-            const float2 hi = __ffma2_rn(ac, f2sub(B2, C2), C2);
-            v = __ffma2_rn(f2(t1.z, t1.w), f2sub(hi, v), v);
-        }
-        fs[k] = v;
+    for (int k = 0; k < QW; ++k) {
+        const float4 t0 = tb[3 * k], t1 = tb[3 * k + 1];
         const float2 c = f2(t0.x, t0.y), sn = f2(t0.z, t0.w);
-        const float2 cv = __fmul2_rn(c, v);
-        s0 = __fadd2_rn(s0, v);
-        sc = __fadd2_rn(sc, cv);
-        ss = __ffma2_rn(sn, v, ss);
-        scc = __ffma2_rn(c, cv, scc);
-        scs = __ffma2_rn(sn, cv, scs);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool left = u == 0 || u == 3; // pulls from x - 1
+            const float2 ax = (u & 1) ? sn : c, ay = (u & 1) ? c : sn;
+            const St *ra = cb + u * aw + k * BW;
+            const float2 C = lds2<St>(ra);
+            const float e = lds1<St>(ra + (left ? -1 : 2));
+            float2 v = left ? lerp_x<true>(C, e, ax) : lerp_x<false>(C, e, ax);
+            if (TWO_D) {
+                const St *rb = pb + u * aw + k * BW;
+                const float2 C2 = lds2<St>(rb);
+                const float e2 = lds1<St>(rb + (left ? -1 : 2));
+                const float2 h = left ? lerp_x<true>(C2, e2, ax) : lerp_x<false>(C2, e2, ax);
+                v = pfma(ay, psub(h, v), v);
+            }
+            fs[4 * k + u] = v;
+        }
+        sums.add(t0, t1, fs + 4 * k);
     }
     if (L.alias) __syncthreads(); // red and sres alias the stage: every warp is done reading it
-    float2 *red2 = reinterpret_cast<float2 *>(red);
-    red2[(0 * G + g) * 32 + lane] = s0;
-    red2[(1 * G + g) * 32 + lane] = sc;
-    red2[(2 * G + g) * 32 + lane] = ss;
-    red2[(3 * G + g) * 32 + lane] = scc;
-    red2[(4 * G + g) * 32 + lane] = scs;
-    __syncthreads();
+    sums.store(reinterpret_cast<float2 *>(red), G, g, lane);
     constexpr bool DD = sizeof(St) == 4; // FP32 storage: FP64-class per-site part
-    if (g < 2) {
-        const int s = g * 32 + lane;
-        if constexpr (DD) pair_site_solve_dd<N>(a, red, G, s, x0 + s < a.nx, sres);
-        else pair_site_solve<N>(a, red, G, s, x0 + s < a.nx, sres);
-    }
-    __syncthreads();
+    quad_site<N, DD, false>(a, red, G, Gs, G, g, lane, blockIdx.x + blockIdx.y, sres,
+                            [&](int s) { return x0 + s < a.nx ? (long long)s : -1ll; });
 
     // pass 2: this warp's shell coefficients, f^eq, relaxation (Eq. discrete-rbe), stores
-    float2 cr[NC], o0, o1, o2;
-    pair_shell_coefficients<N, DD>(a, r, sres, lane, cr, o0, o1, o2);
-    const float2 no1 = f2(-o1.x, -o1.y), no2 = f2(-o2.x, -o2.y);
-    unsigned rng = mix32(unsigned(y * a.nx + xl) * 64u + unsigned(g) ^ mix32(__ldcg(a.ctr) * 0x9E3779B9u + 1u));
-    St *ob = reinterpret_cast<St *>(a.fout) + (long long)i0 * S + (long long)y * a.nx + (act ? xl : 0);
+    float2 cf[NC], o[3];
+    quad_shell<N, DD>(a, r, r, q, Gs, sres, red, lane, cf, o);
+    QuadBits rng = quad_seed(unsigned(y * a.nx + xl), unsigned(g), seed);
+    const long long Sb = S * (long long)sizeof(St), KS = K4 * Sb;
+    char *ob = reinterpret_cast<char *>(a.fout) + i0 * Sb + ((long long)y * a.nx + (act ? xl : 0)) * int(sizeof(St));
 #pragma unroll
-    for (int k = 0; k < PP; ++k) {
-        const float4 t0 = tb[k * PQ];                                      // (c,c,s,s)
-        const float2 wq = *reinterpret_cast<const float2 *>(tb + k * PQ + 2); // (w', w')
-        const float2 c = f2(t0.x, t0.y), sn = f2(t0.z, t0.w);
-        const float2 cc = __fmul2_rn(c, c), cs = __fmul2_rn(c, sn);
-        float2 pe = __ffma2_rn(cr[1], c, cr[0]);
-        pe = __ffma2_rn(cr[2], sn, pe);
-        pe = __ffma2_rn(cr[3], cc, pe);
-        pe = __ffma2_rn(cr[4], cs, pe);
-        if (N == 3) {
-            pe = __ffma2_rn(cr[NC - 2], __fmul2_rn(c, cc), pe);
-            pe = __ffma2_rn(cr[NC - 1], __fmul2_rn(sn, cc), pe);
-        }
-        const float2 feq = __fmul2_rn(wq, pe);
-        const float2 om = __ffma2_rn(no2, sn, __ffma2_rn(no1, c, o0));
-        const unsigned rb = next_bits2(rng);
-        if constexpr (sizeof(St) == 4) {
-            const float2 out = relax_pair_sr(fs[k], om, feq, rb);
-            if (act) *reinterpret_cast<float2 *>(ob + (long long)k * S) = out;
-        } else {
-            const float2 out = __ffma2_rn(om, f2sub(feq, fs[k]), fs[k]);
-            if (act) st2_rs<St>(ob + (long long)k * S, out, rb);
+    for (int k = 0; k < QW; ++k) {
+        float2 feq[4], om[4];
+        quad_equilibrium<N>(cf, o, tb + 3 * k, feq, om);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            char *p = ob + (k * Sb + u * KS);
+            const float2 f = fs[4 * k + u];
+            if constexpr (sizeof(St) == 4) {
+                const float2 out = quad_relax_sr(f, om[u], feq[u], rng.next());
+                if (act) *reinterpret_cast<float2 *>(p) = out;
+            } else {
+                const unsigned d = cvt2_rs<St>(pfma(om[u], psub(feq[u], f), f), rng.next());
+                if (act) *reinterpret_cast<unsigned *>(p) = d;
+            }
         }
     }
     __syncthreads();
@@ -230,7 +193,7 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
 
 // FP32 storage: the launch bounds of the other two-sites-per-lane kernels.
 template <class St, int N, int PP, bool TWO_D>
-__global__ void __launch_bounds__(kMaxWarps * 32, PP <= 16 ? 2 : 1)
+__global__ void __maxnreg__(PP <= 16 ? 64 : (PP == 24 ? 104 : 128))
     rlbm_pair_tma_kernel(const __grid_constant__ PairTmaArgs ta)
 {
     pair_tma_body<St, N, PP, TWO_D>(ta);
@@ -240,7 +203,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, PP <= 16 ? 2 : 1)
 // warps (the 2048^2 N = 2 K = 48 tiling, 54 KB of shared memory with the aliased
 // sums) share an SM.
 template <class St, int N, int PP, bool TWO_D>
-__global__ void __maxnreg__(PP <= 16 ? 56 : 128) rlbm_pair_tma_kernel16(const __grid_constant__ PairTmaArgs ta)
+__global__ void __maxnreg__(PP <= 16 ? 56 : (PP == 24 ? 80 : 96)) rlbm_pair_tma_kernel16(const __grid_constant__ PairTmaArgs ta)
 {
     pair_tma_body<St, N, PP, TWO_D>(ta);
 }
@@ -256,7 +219,7 @@ static cudaError_t launch_pair_tma_np(bool two_d, dim3 grid, dim3 block, size_t 
         k = two_d ? rlbm_pair_tma_kernel<St, N, PP, true> : rlbm_pair_tma_kernel<St, N, PP, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (bps) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k, int(block.x * block.y), smem);
+    if (bps) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k, int(block.x * block.y * block.z), smem);
     k<<<grid, block, smem, st>>>(ta);
     return cudaGetLastError();
 }

@@ -314,6 +314,124 @@ RLBM_HDX bool stat_solve(double n, double e, double g, int stat, double &eta, do
     return ok;
 }
 
+// ---- the FP32-storage Fermi-Dirac solve with few FP64 operations ---------------------
+// FP64 runs at 1/64 of the FP32 rate, so what matters is the number of FP64 operations a
+// site costs.  The accelerated series of phi_1 .. phi_4 become polynomials in z = e^-|eta|
+// evaluated by Horner's rule (one FMA per term and order; weights formed at compile time),
+// the equation is solved to about 1e-6 by FP32 Newton steps and finished by one FP64 step
+// whose residual needs no logarithm: with
+//   q = phi_3^2 4 n^3 / (phi_2^3 2 pi g e^2)   (q = 1 at the root)
+// the equation is H = 1/2 ln q = 0, and q - 1 is of the order of the FP32 error, so
+// ln q = d - d^2/2 + d^3/3 (d = q - 1) to 1e-24.  Its slope is needed in FP32 only.
+struct StatPoly {
+    double c[4][kStatTermsShort]; // w_k / (k + 1)^s, s = 1..4
+};
+constexpr int kStatTermsF32 = 12; // error below 2 (3 + sqrt 8)^-12 ~ 1e-9 of the first term
+struct StatPolyF {
+    float c[3][kStatTermsF32];
+};
+constexpr StatPoly stat_poly()
+{
+    StatPoly p{};
+    const StatSeriesTab t = stat_series_tab(kStatTermsShort);
+    for (int k = 0; k < kStatTermsShort; ++k) {
+        double v = t.w[k];
+        for (int s = 0; s < 4; ++s) p.c[s][k] = v = v / (k + 1.0);
+    }
+    return p;
+}
+constexpr StatPolyF stat_poly_f()
+{
+    StatPolyF p{};
+    const StatSeriesTab t = stat_series_tab(kStatTermsF32);
+    for (int k = 0; k < kStatTermsF32; ++k) {
+        double v = t.w[k];
+        for (int s = 0; s < 3; ++s) {
+            v = v / (k + 1.0);
+            p.c[s][k] = float(v);
+        }
+    }
+    return p;
+}
+#ifdef __CUDACC__
+static __constant__ StatPoly kStatPolyDev = stat_poly();
+static __constant__ StatPolyF kStatPolyFDev = stat_poly_f();
+#endif
+static constexpr StatPoly kStatPolyHost = stat_poly();
+static constexpr StatPolyF kStatPolyFHost = stat_poly_f();
+
+// (eta, T) and phi_1 .. phi_4 of the Fermi-Dirac equilibrium with density n and energy
+// density e (as stat_solve with the FP32-storage rule); x0: a start (NaN: none).  False
+// where the FP32 steps do not lead to a small FP64 step: the caller then uses stat_solve.
+RLBM_HD bool stat_solve_fd_short(double n, double e, double g, double x0, double &eta, double &T, double *phi)
+{
+#ifdef __CUDA_ARCH__
+    const StatPoly &P = kStatPolyDev;
+    const StatPolyF &F = kStatPolyFDev;
+#else
+    const StatPoly &P = kStatPolyHost;
+    const StatPolyF &F = kStatPolyFHost;
+#endif
+    const double twopi = 6.283185307179586477, pi2 = 9.8696044010893586188;
+    // H = ln phi_3 - 3/2 ln phi_2 - L, L = ln(e sqrt(2 pi g) / (2 n^1.5))
+    const float L = logf(float(e)) - 1.5f * logf(float(n)) + 0.5f * logf(float(twopi * g)) - 0.69314718f;
+    float x = float(x0);
+    if (!(x > -60.f && x < 700.f)) x = -2.f * L;
+    bool done = false;
+    for (int it = 0; it < 12 && !done; ++it) {
+        const float z = expf(-fabsf(x));
+        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        for (int k = kStatTermsF32 - 1; k >= 0; --k) {
+            a1 = a1 * z + F.c[0][k];
+            a2 = a2 * z + F.c[1][k];
+            a3 = a3 * z + F.c[2][k];
+        }
+        float p1f = a1 * z, p2f = a2 * z, p3f = a3 * z;
+        if (x > 0.f) { // inversion identity
+            p1f += x;
+            p2f = 0.5f * x * x + float(pi2 / 6.0) - p2f;
+            p3f += x * (x * x * float(1.0 / 6.0) + float(pi2 / 6.0));
+        }
+        const float d = (logf(p3f) - 1.5f * logf(p2f) - L) / (p2f / p3f - 1.5f * p1f / p2f);
+        x -= d;
+        done = fabsf(d) <= 1e-4f * (1.f + fabsf(x)); // the next step would be at rounding level
+    }
+    if (!done) return false;
+    double xd = double(x), dx = 0.0, a[4];
+    done = false;
+    for (int it = 0; it < 4 && !done; ++it) { // one step, or two for a strongly degenerate gas
+        xd += dx;
+        const double z = exp(-fabs(xd));
+        for (int s = 0; s < 4; ++s) a[s] = P.c[s][kStatTermsShort - 1];
+        for (int k = kStatTermsShort - 2; k >= 0; --k)
+            for (int s = 0; s < 4; ++s) a[s] = a[s] * z + P.c[s][k];
+        for (int s = 0; s < 4; ++s) a[s] *= z;
+        if (xd > 0.0) {
+            const double x2 = xd * xd;
+            a[0] += xd;
+            a[1] = 0.5 * x2 + pi2 / 6.0 - a[1];
+            a[2] += xd * (x2 * (1.0 / 6.0) + pi2 / 6.0);
+            a[3] = x2 * (x2 * (1.0 / 24.0) + pi2 / 12.0) + 7.0 * pi2 * pi2 / 360.0 - a[3];
+        }
+        const double d = (a[2] * a[2]) * (4.0 * n * n * n) / ((a[1] * a[1] * a[1]) * (twopi * g * e * e)) - 1.0;
+        if (!(fabs(d) < 0.1)) return false;
+        const double H = 0.5 * d * (1.0 - d * (0.5 - d * (1.0 / 3.0)));
+        const float b1 = float(a[0]), b2 = float(a[1]), b3 = float(a[2]);
+        dx = -H / double(b2 / b3 - 1.5f * b1 / b2);
+        done = fabs(dx) <= 3e-6 * (1.0 + fabs(xd));
+    }
+    if (!done) return false;
+    eta = xd + dx;
+    // phi_s(eta) from phi_s(x) by Taylor's formula, phi_0 = 1 / (1 + e^-x)
+    const double p0 = double(1.f / (1.f + expf(-float(xd))));
+    phi[0] = a[0] + dx * p0;
+    phi[1] = a[1] + dx * (a[0] + 0.5 * dx * p0);
+    phi[2] = a[2] + dx * (a[1] + 0.5 * dx * a[0]);
+    phi[3] = a[3] + dx * (a[2] + 0.5 * dx * a[1]);
+    T = sqrt(n / (twopi * g * phi[1]));
+    return true;
+}
+
 // eta of the equilibrium with density n at temperature T: phi_2(eta) = n / (2 pi g T^2).
 RLBM_HDX bool stat_fugacity(double n, double T, double g, int stat, double &eta)
 {

@@ -688,7 +688,7 @@ bool pair_bulk_possible(const rlbm_t *h)
 bool quad_possible(const rlbm_t *h, int P)
 {
     int gs = 0, ng = 0;
-    return h->prec != RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && !h->stat &&
+    return h->prec != RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && (!h->stat || h->prec == RLBM_FP32) &&
            (P == 8 || P == 12 || P == 16 || P == 24 || P == 32) && h->K % P == 0 &&
            group_tiling(h->N, h->K, P, gs, ng) && ng == 1;
 }
@@ -699,6 +699,11 @@ cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
     const bool two_d = h->grid.ny > 1;
     const size_t smem = rlbmk::pair_smem_bytes(h->N, h->G, false, int(storage_size(h->prec)), two_d);
     cudaError_t e;
+    if (h->stat) {
+        e = rlbmk::launch_quad_stat_f32(h->N, h->P, map, two_d, block, smem, h->stream, a);
+        if (e == cudaSuccess) ++h->launches;
+        return e;
+    }
     switch (h->prec) {
     case RLBM_FP32: e = rlbmk::launch_quad_f32(h->N, h->P, map, two_d, block, smem, h->stream, a); break;
     case RLBM_FP16_DEV:
@@ -1279,6 +1284,10 @@ int rlbm_quantum_solve(double n, double e, double g, int statistics, double eta0
     *eta = std::nan("");
     *T = std::nan("");
     if ((statistics != 1 && statistics != -1) || !(g > 0.0)) return 0;
+    double phi[4];
+    if (fp32_storage && statistics > 0 && n > 0.0 && e > 0.0 &&
+        rlbmk::stat_solve_fd_short(n, e, g, eta0, *eta, *T, phi))
+        return 1;
     return rlbmk::stat_solve(n, e, g, statistics, *eta, *T, eta0, nullptr, 0, fp32_storage ? 1e-5 : 1e-10) ? 1 : 0;
 }
 

@@ -4,6 +4,9 @@ rows for ny > 1 and any nx, with an odd number of rows; 32 apart for ny = 1), gr
 than a tile, one cell or one row beyond a tile, both boundary conditions, one, two and four
 warps per shell, N = 2 and 3.
 
+Fermi-Dirac and
+Bose-Einstein: the FP32 bound, on rows the statistics' own tests do not have.
+
 FP32 storage: the bound of the other FP32 parity tests (FP32 arithmetic per population, a few
 steps).  16-bit storage: stochastic rounding adds at most one unit in the last place per value
 and step (2^-10 for FP16, 2^-7 for BF16), which the moments average over the populations; the
@@ -54,6 +57,24 @@ def test_fp32_any_row_length(nx, ny, bcx, bcy, N, K, P):
     for kind in ("per-tile", "pair") if nx % 2 == 0 else ("per-tile",):
         f, _, ref, _ = run_both(nx, ny, N, K, 2.5, "fp32", bcx, bcy, P, kind, 5)
         assert relerr(f, ref) < FP32_TOL, kind
+
+
+@pytest.mark.parametrize("stat", ["fd", "be"])
+@pytest.mark.parametrize("N,K,P,nx,ny", [(2, 16, 8, 9, 3), (3, 12, 12, 33, 2), (2, 24, 24, 35, 1)])
+def test_fp32_statistics_any_row_length(stat, N, K, P, nx, ny):
+    from oracle import statistics as S
+    eps, g = {"fd": S.FD, "be": S.BE}[stat], 1.0
+    fl = W.random_fields(nx, ny, seed=5, beta_max=0.2)
+    fl.n[:] *= 0.5  # fugacities below 1 for the Bose-Einstein runs
+    q = O.Quadrature(N, K)
+    ref = S.run(q, S.init(q, fl.n, fl.T, fl.bx, fl.by, eps, g), 3.0, 3, OUT, PER, eps, g)
+    with R.Simulation(nx, ny, N, K, 3.0, "fp32", OUT, PER) as sim:
+        sim.set_statistics(stat, g)
+        sim.set_tiling(P, "per-tile")
+        sim.init_fields(fl)
+        sim.step(3)
+        sim.sync()
+        assert relerr(sim.get_populations().astype(np.float64), ref) < FP32_TOL
 
 
 @pytest.mark.parametrize("precision,tol", [("fp16n", 2.0 ** -10), ("fp16", 2.0 ** -10), ("bf16n", 2.0 ** -7), ("bf16", 2.0 ** -7)])

@@ -693,6 +693,23 @@ bool quad_possible(const rlbm_t *h, int P)
            group_tiling(h->N, h->K, P, gs, ng) && ng == 1;
 }
 
+// FP64 storage: the same conditions (P up to 32: the populations are kept in registers).
+bool quad64_possible(const rlbm_t *h)
+{
+    const int P = h->P;
+    return h->prec == RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && !h->stat && h->R == 1 &&
+           (P == 8 || P == 12 || P == 16 || P == 24 || P == 32) && h->K % P == 0;
+}
+
+cudaError_t launch_quad64(rlbm_t *h, const rlbmk::KernelArgs &a)
+{
+    const dim3 block(32, h->Gs, h->N + 1);
+    cudaError_t e = h->N == 2 ? rlbmk::launch_quad_f64_n2(h->P, block, h->stream, a)
+                              : rlbmk::launch_quad_f64_n3(h->P, block, h->stream, a);
+    if (e == cudaSuccess) ++h->launches;
+    return e;
+}
+
 cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
 {
     const dim3 block(32, h->Gs, h->N + 1);
@@ -808,6 +825,7 @@ cudaError_t launch_step(rlbm_t *h, int from)
     }
     const int map = h->grid.ny > 1 ? rlbmk::kMapCol : rlbmk::kMapSplit; // for any nx
     if (quad_possible(h, h->P)) return launch_quad(h, map, a);
+    if (quad64_possible(h)) return launch_quad64(h, a);
     return launch(h, rlbmk::MODE_STEP, a);
 }
 

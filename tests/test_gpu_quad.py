@@ -4,7 +4,7 @@ rows for ny > 1 and any nx, with an odd number of rows; 32 apart for ny = 1), gr
 than a tile, one cell or one row beyond a tile, both boundary conditions, one, two and four
 warps per shell, N = 2 and 3.
 
-Fermi-Dirac and
+FP64 storage (csrc/rlbm_quad64.cuh): the bound of the other FP64 parity tests.  Fermi-Dirac and
 Bose-Einstein: the FP32 bound, on rows the statistics' own tests do not have.
 
 FP32 storage: the bound of the other FP32 parity tests (FP32 arithmetic per population, a few
@@ -57,6 +57,14 @@ def test_fp32_any_row_length(nx, ny, bcx, bcy, N, K, P):
     for kind in ("per-tile", "pair") if nx % 2 == 0 else ("per-tile",):
         f, _, ref, _ = run_both(nx, ny, N, K, 2.5, "fp32", bcx, bcy, P, kind, 5)
         assert relerr(f, ref) < FP32_TOL, kind
+
+
+@pytest.mark.parametrize("nx,ny,bcx,bcy", [(1, 1, PER, PER), (31, 2, PER, PER), (33, 5, OUT, OUT), (63, 1, OUT, PER),
+                                           (64, 4, PER, PER), (97, 3, PER, OUT)])
+@pytest.mark.parametrize("N,K,P", [(2, 8, 8), (2, 24, 12), (3, 32, 8), (3, 16, 16), (2, 48, 24), (3, 64, 32)])
+def test_fp64_any_row_length(nx, ny, bcx, bcy, N, K, P):
+    f, m, ref, mac = run_both(nx, ny, N, K, 2.5, "fp64", bcx, bcy, P, "per-tile", 5)
+    assert relerr(f, ref) < 1e-12 and relerr(m, mac) < 1e-12
 
 
 @pytest.mark.parametrize("stat", ["fd", "be"])

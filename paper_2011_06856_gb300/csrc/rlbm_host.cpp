@@ -1379,6 +1379,22 @@ rlbm_status rlbm_step(rlbm_t *h, int nsteps)
     if (!h) return fail(nullptr, RLBM_ERR_ARG, "NULL handle");
     if (nsteps < 0) return fail(h, RLBM_ERR_ARG, "nsteps must be >= 0");
     int left = nsteps;
+    // free streaming of a thin grid: up to kFreeSteps steps per launch (rlbm_free.cu); grids
+    // of more rows, 16-bit storage and the on-lattice shifts step one launch at a time
+    const bool free_thin = std::isinf(h->tau) && h->grid.ny <= rlbmk::kFreeRows && storage_size(h->prec) >= 4 &&
+                           !h->q.onlat && !h->stall_next;
+    while (free_thin && left > 0) {
+        const int n = std::min(left, rlbmk::kFreeSteps);
+        rlbmk::KernelArgs a = h->base;
+        a.fin = buffer(h, h->cur);
+        a.fout = buffer(h, 1 - h->cur);
+        cudaError_t e = rlbmk::launch_free(h->prec == RLBM_FP64, h->N, h->npop, n, h->stream, a);
+        if (e != cudaSuccess) return cuda_fail(h, e, "free-streaming kernel");
+        ++h->launches;
+        h->cur = 1 - h->cur;
+        h->steps += n;
+        left -= n;
+    }
     while (left >= kGraphSteps) {
         rlbm_status st = ensure_graph(h, h->cur);
         if (st) return st;

@@ -31,6 +31,8 @@
 
 #include "rlbm_pair.cuh"
 
+#include <type_traits>
+
 namespace rlbmk {
 
 // ---- the per-site part, for the tile's 64 sites ------------------------------------
@@ -518,6 +520,10 @@ template <bool B> struct QuadTag {
     static constexpr bool value = B;
 };
 
+// v, which is the same in every lane, as a value the compiler knows to be (a shuffle from a
+// fixed lane): what follows from it runs on the uniform pipe.
+__device__ __forceinline__ int warp_uniform(unsigned v) { return int(__shfl_sync(0xffffffffu, v, 0)); }
+
 // The place of a CTA's 64 sites in the grid.
 template <int MAP> struct QuadTile {
     static constexpr bool COL = MAP == kMapCol, SPLIT = MAP == kMapSplit;
@@ -546,62 +552,79 @@ template <int MAP> struct QuadTile {
 // The bilinear pull (Eqs. streaming, interpolation) of half a quad: populations u = H and
 // H + 2.  EDGE: the tile touches the x boundary, a lane's neighbours are at its own
 // wrapped or clamped offsets; else they are at fixed offsets from the centre.
+//
+// Addresses: base, the rows and the quad are the same for all lanes of a warp, so a
+// population's row is a uniform 64-bit address (formed on the uniform pipe) and a lane adds
+// its 32-bit offset in the load itself; 64-bit address arithmetic per lane and row took
+// about a quarter of the first pass's instructions and 16 registers.
 template <class St, int MAP, bool TWO_D, bool EDGE> struct QuadPull {
     static constexpr bool COL = MAP == kMapCol, SPLIT = MAP == kMapSplit;
     static_assert(!COL || TWO_D, "two rows per lane need ny > 1");
     struct Half {
         float2 C[2], B[2], C2[2], B2[2]; // kMapRow: the neighbour in B.x, B2.x; kMapCol: the pull row in C2.x, B2.x
     };
-    const char *pa, *pb, *pu, *pd; // rows y, y + 1 (kMapCol), the pull rows of the upward and downward populations
-    int em, ep, em2, ep2, ec2;     // offsets (elements) of the left and right neighbours, of the second site
-    // base: the populations' first byte in the input buffer
+    static constexpr int ES = int(sizeof(St));
+    using Off = std::conditional_t<EDGE, long long, unsigned>; // a lane's byte offset from the tile corner's column
+    const char *pa, *pb, *pu, *pd; // at the tile's first column (uniform): rows y, y + 1 (kMapCol), the pull rows of the
+                                   // upward and downward populations
+    Off oc, om, op, oc2, om2, op2; // the lane's site, its left and right neighbours; the second site's (kMapSplit)
+    // base: the populations' first byte in the input buffer, the same for the warp
     __device__ __forceinline__ QuadPull(const KernelArgs &a, const QuadTile<MAP> &t, const char *base)
     {
-        constexpr int ES = int(sizeof(St)), RIGHT = MAP == kMapRow ? 2 : 1;
+        constexpr int RIGHT = MAP == kMapRow ? 2 : 1;
         const int yb = COL ? (t.y + 1 < a.ny ? t.y + 1 : bc_index(a.ny, a.ny, a.bcy)) : t.y;
         const int yu = TWO_D ? bc_index(t.y - 1, a.ny, a.bcy) : t.y;
         const int yd = TWO_D ? (COL ? bc_any(t.y + 2, a.ny, a.bcy) : bc_index(t.y + 1, a.ny, a.bcy)) : t.y;
-        auto row = [&](int y) { return base + ((long long)y * a.nx + t.x) * ES; };
+        auto row = [&](int y) { return base + ((long long)y * a.nx + t.x0) * ES; };
         pa = row(t.y);
         pb = row(yb);
         pu = row(yu);
         pd = row(yd);
-        em = EDGE ? bc_index(t.x - 1, a.nx, a.bcx) - t.x : -1;
-        ep = EDGE ? bc_index(t.x + RIGHT, a.nx, a.bcx) - t.x : RIGHT;
-        em2 = SPLIT ? (EDGE ? bc_index(t.x2 - 1, a.nx, a.bcx) - t.x : 31) : 0;
-        ep2 = SPLIT ? (EDGE ? bc_index(t.x2 + 1, a.nx, a.bcx) - t.x : 33) : 0;
-        ec2 = SPLIT ? (EDGE ? t.x2 - t.x : 32) : 0;
+        auto off = [&](int x) { return Off(x - t.x0) * ES; };
+        oc = off(t.x);
+        om = off(EDGE ? bc_index(t.x - 1, a.nx, a.bcx) : t.x - 1);
+        op = off(EDGE ? bc_index(t.x + RIGHT, a.nx, a.bcx) : t.x + RIGHT);
+        oc2 = off(t.x2);
+        om2 = SPLIT ? off(EDGE ? bc_index(t.x2 - 1, a.nx, a.bcx) : t.x2 - 1) : 0;
+        op2 = SPLIT ? off(EDGE ? bc_index(t.x2 + 1, a.nx, a.bcx) : t.x2 + 1) : 0;
     }
     // off: bytes to population u = 0 of the quad, KS: to its next population
     template <int H> __device__ __forceinline__ void load(Half &b, long long off, long long KS) const
     {
-        auto at = [](const char *p) { return reinterpret_cast<const St *>(p); };
+        constexpr int RIGHT = MAP == kMapRow ? 2 : 1;
+        // interior: fixed distances from the lane's own offset; a left neighbour is one element
+        // before the row's address, so that the 32-bit offset stays positive
+        auto centre = [&](const char *row) { return reinterpret_cast<const St *>(row + oc); };
+        auto beside = [&](const char *row, bool left) {
+            if (EDGE) return reinterpret_cast<const St *>(row + (left ? om : op));
+            return reinterpret_cast<const St *>((row + (left ? -ES : RIGHT * ES)) + oc);
+        };
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
             constexpr bool L0 = H == 0;
             const int u = H + 2 * v;
             const bool left = L0 ? v == 0 : v == 1; // u = 0 and u = 3 pull from x - 1
-            const int e = left ? em : ep;
             const long long o = off + u * KS;
-            const St *ra = at(pa + o);
+            const char *ra = pa + o;
             if (MAP == kMapRow) {
-                b.C[v] = PIo<St>::ld2(ra);
-                b.B[v].x = PIo<St>::ld1(ra + e);
+                b.C[v] = PIo<St>::ld2(centre(ra));
+                b.B[v].x = PIo<St>::ld1(beside(ra, left));
                 if (TWO_D) {
-                    const St *rr = at((u < 2 ? pu : pd) + o);
-                    b.C2[v] = PIo<St>::ld2(rr);
-                    b.B2[v].x = PIo<St>::ld1(rr + e);
+                    const char *rr = (u < 2 ? pu : pd) + o;
+                    b.C2[v] = PIo<St>::ld2(centre(rr));
+                    b.B2[v].x = PIo<St>::ld1(beside(rr, left));
                 }
             } else if (SPLIT) {
-                b.C[v] = f2(PIo<St>::ld1(ra), PIo<St>::ld1(ra + ec2));
-                b.B[v] = f2(PIo<St>::ld1(ra + e), PIo<St>::ld1(ra + (left ? em2 : ep2)));
+                auto at = [&](Off x) { return PIo<St>::ld1(reinterpret_cast<const St *>(ra + x)); };
+                b.C[v] = f2(at(oc), at(oc2));
+                b.B[v] = EDGE ? f2(at(left ? om : op), at(left ? om2 : op2))
+                              : f2(PIo<St>::ld1(beside(ra, left)), PIo<St>::ld1(beside(ra, left) + 32));
             } else {
-                const St *rb = at(pb + o);
-                const St *rr = at((u < 2 ? pu : pd) + o);
-                b.C[v] = f2(PIo<St>::ld1(ra), PIo<St>::ld1(rb));
-                b.B[v] = f2(PIo<St>::ld1(ra + e), PIo<St>::ld1(rb + e));
-                b.C2[v].x = PIo<St>::ld1(rr);
-                b.B2[v].x = PIo<St>::ld1(rr + e);
+                const char *rb = pb + o, *rr = (u < 2 ? pu : pd) + o;
+                b.C[v] = f2(PIo<St>::ld1(centre(ra)), PIo<St>::ld1(centre(rb)));
+                b.B[v] = f2(PIo<St>::ld1(beside(ra, left)), PIo<St>::ld1(beside(rb, left)));
+                b.C2[v].x = PIo<St>::ld1(centre(rr));
+                b.B2[v].x = PIo<St>::ld1(beside(rr, left));
             }
         }
     }
@@ -637,12 +660,16 @@ template <class St, int MAP, bool TWO_D, bool EDGE> struct QuadPull {
 // The relaxed populations of a quad into the output (Eq. discrete-rbe), rounded
 // stochastically.  base: as in QuadPull, in the output buffer.
 template <class St, int MAP> struct QuadOut {
-    char *pa, *pb; // first and second site (kMapRow: one paired store)
+    char *pa, *pb;    // rows of the first and second site at the tile's first column (uniform)
+    unsigned oa, ob;  // the lane's byte offsets (kMapRow: one paired store)
     bool act0, act1;
     __device__ __forceinline__ QuadOut(const KernelArgs &a, const QuadTile<MAP> &t, char *base)
     {
-        pa = base + ((long long)t.y * a.nx + t.x) * int(sizeof(St));
-        pb = base + ((long long)(t.y + (MAP == kMapCol && t.act1 ? 1 : 0)) * a.nx + t.x2) * int(sizeof(St));
+        constexpr unsigned ES = sizeof(St);
+        pa = base + ((long long)t.y * a.nx + t.x0) * ES;
+        pb = pa + (MAP == kMapCol && t.y + 1 < a.ny ? (long long)a.nx * ES : 0ll);
+        oa = unsigned(t.x - t.x0) * ES;
+        ob = unsigned(t.x2 - t.x0) * ES;
         act0 = t.act0;
         act1 = t.act1;
     }
@@ -655,18 +682,18 @@ template <class St, int MAP> struct QuadOut {
             if constexpr (sizeof(St) == 4) {
                 const float2 out = quad_relax_sr(f[u], om[u], feq[u], rng.next());
                 if (MAP == kMapRow) {
-                    if (act0) *reinterpret_cast<float2 *>(pa + o) = out;
+                    if (act0) *reinterpret_cast<float2 *>(pa + o + oa) = out;
                 } else {
-                    if (act0) *reinterpret_cast<float *>(pa + o) = out.x;
-                    if (act1) *reinterpret_cast<float *>(pb + o) = out.y;
+                    if (act0) *reinterpret_cast<float *>(pa + o + oa) = out.x;
+                    if (act1) *reinterpret_cast<float *>(pb + o + ob) = out.y;
                 }
             } else {
                 const unsigned d = cvt2_rs<St>(pfma(om[u], psub(feq[u], f[u]), f[u]), rng.next());
                 if (MAP == kMapRow) {
-                    if (act0) *reinterpret_cast<unsigned *>(pa + o) = d;
+                    if (act0) *reinterpret_cast<unsigned *>(pa + o + oa) = d;
                 } else {
-                    if (act0) *reinterpret_cast<unsigned short *>(pa + o) = (unsigned short)d;
-                    if (act1) *reinterpret_cast<unsigned short *>(pb + o) = (unsigned short)(d >> 16);
+                    if (act0) *reinterpret_cast<unsigned short *>(pa + o + oa) = (unsigned short)d;
+                    if (act1) *reinterpret_cast<unsigned short *>(pb + o + ob) = (unsigned short)(d >> 16);
                 }
             }
         }
@@ -682,7 +709,8 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
     constexpr int NC = 2 * N + 1, QW = PP / 4;
     constexpr bool DD = sizeof(St) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x, q = threadIdx.y, Gs = blockDim.y, r = threadIdx.z, K4 = a.K >> 2;
+    const int lane = threadIdx.x, Gs = blockDim.y, K4 = a.K >> 2;
+    const int q = warp_uniform(threadIdx.y), r = warp_uniform(threadIdx.z);
     const int g = r * Gs + q, G = Gs * (N + 1);
     const int i0 = r * a.K + q * QW; // population u = 0 of the warp's first quad
     const QuadTile<MAP> t(a, blockIdx.x, blockIdx.y, lane);
@@ -741,144 +769,6 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
     }
     __syncthreads();
     if (g == 0 && lane == 0) advance_launch_counter(a.ctr, gridDim.x * gridDim.y);
-}
-
-// ---- many angles (FP32 storage) -------------------------------------------------------
-//
-// K beyond one group of populations per warp (K = 600, N = 3: 2400 populations, 614 KB for
-// 64 sites) fits no CTA.  A cluster of (N + 1) CS CTAs holds a tile: CTA (r, c) streams
-// quads [c K4 / CS, (c + 1) K4 / CS) of shell r and parks f* in its shared memory between
-// the passes (1 KB per quad; 75 KB for K = 600, so that two CTAs share an SM and one
-// computes while the other loads).  The CTAs write their 5 x 64 angular sums into one
-// another's shared memory (no reads: nothing waits for a remote load) and each forms the
-// per-site part of all 64 sites.  Populations
-// are read and written once; parking f* in the output buffer between the passes
-// (rlbm_pair_groups_kernel) moved 1.5 to 1.9 times the bytes.
-// Warps take quads q, q + Gs, ..: every K4 and CS work.
-template <int N, int MAP, bool TWO_D>
-__global__ void __launch_bounds__(kQuadClusterWarps * 32, 2) rlbm_quad_cluster_kernel(const KernelArgs a)
-{
-    constexpr int NC = 2 * N + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x, q = threadIdx.y, Gs = blockDim.y, K4 = a.K >> 2;
-    const int CL = a.cluster, CS = CL / (N + 1);
-    const int rank = blockIdx.x % CL, r = rank / CS, c = rank % CS;
-    const int j0 = c * K4 / CS, j1 = (c + 1) * K4 / CS; // this CTA's quads of shell r
-    const QuadTile<MAP> t(a, blockIdx.x / CL, blockIdx.y, lane);
-    float *red = reinterpret_cast<float *>(smem_raw); // every CTA's sums [5][CL][64]
-    float *own = red + 5 * CL * kPairSites;           // this CTA's warps' sums [5][Gs][64]
-    float *sres = own + 5 * Gs * kPairSites;          // [pair_site_rows(N)][64]
-    float2 *park = reinterpret_cast<float2 *>(sres + pair_site_rows(N) * kPairSites) + lane; // [quads][4][32]
-    const float4 *tb = reinterpret_cast<const float4 *>(a.quadtab) + size_t(r) * K4 * 3;
-    const unsigned seed = __ldcg(a.ctr);
-    const long long Sb = a.S * 4ll, KS = K4 * Sb, base = (long long)r * a.K * Sb;
-
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); // waited for before the exchange
-    QuadSums sums = quad_sums_zero();
-    auto pass1 = [&](auto edge_tag) {
-        using Pull = QuadPull<float, MAP, TWO_D, decltype(edge_tag)::value>;
-        const Pull p(a, t, reinterpret_cast<const char *>(a.fin) + base);
-        // the loads run a quad ahead of the arithmetic
-        typename Pull::Half b[2][2];
-        auto load = [&](int v, int j) {
-            if (j >= j1) return;
-            p.template load<0>(b[v][0], j * Sb, KS);
-            p.template load<1>(b[v][1], j * Sb, KS);
-        };
-        auto pull = [&](int v, int j) {
-            if (j >= j1) return;
-            const float4 t0 = __ldg(tb + 3 * j), t1 = __ldg(tb + 3 * j + 1);
-            float2 f[4];
-            Pull::template pull<0>(b[v][0], t0, f);
-            Pull::template pull<1>(b[v][1], t0, f);
-            sums.add(t0, t1, f);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) park[((j - j0) * 4 + u) * 32] = f[u];
-        };
-        int j = j0 + q;
-        load(0, j);
-#pragma unroll 1
-        for (; j < j1; j += 2 * Gs) {
-            load(1, j + Gs);
-            pull(0, j);
-            load(0, j + 2 * Gs);
-            pull(1, j + Gs);
-        }
-    };
-    if (t.interior(a)) pass1(QuadTag<false>{});
-    else pass1(QuadTag<true>{});
-    sums.store(reinterpret_cast<float2 *>(own), Gs, q, lane);
-    // every CTA has begun: its shared memory may be written to
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    __syncthreads();
-    // this CTA's sums, written into every CTA of the cluster
-    for (int e = q * 32 + lane; e < 5 * kPairSites; e += Gs * 32) {
-        const int u = e >> 6, s = e & 63;
-        const float *p = own + u * Gs * kPairSites + s;
-        float v = p[0];
-        for (int w = 1; w < Gs; ++w) v += p[w * kPairSites];
-        const unsigned at = sptr(red + (u * CL + rank) * kPairSites + s);
-        for (int to = 0; to < CL; ++to) {
-            unsigned dst;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(at), "r"(to));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(v) : "memory");
-        }
-    }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    quad_site<N, true, false>(a, red, CL, CS, Gs, q, lane, blockIdx.x + blockIdx.y, sres,
-                              [&](int s) { return t.site(a, s); });
-
-    float2 cf[NC], o[3];
-    quad_shell<N, true>(a, r, 0, q, Gs, sres, red, lane, cf, o);
-    QuadBits rng = quad_seed(unsigned(t.y * a.nx + t.x), unsigned(rank * Gs + q), seed);
-    const QuadOut<float, MAP> out(a, t, reinterpret_cast<char *>(a.fout) + base);
-#pragma unroll 1
-    for (int j = j0 + q; j < j1; j += Gs) {
-        const float4 tq[3] = {__ldg(tb + 3 * j), __ldg(tb + 3 * j + 1),
-                              N == 3 ? __ldg(tb + 3 * j + 2) : make_float4(0.f, 0.f, 0.f, 0.f)};
-        float2 f[4], feq[4], om[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) f[u] = park[((j - j0) * 4 + u) * 32];
-        quad_equilibrium<N>(cf, o, tq, feq, om);
-        out.store(j * Sb, KS, f, feq, om, rng);
-    }
-    __syncthreads();
-    if (q == 0 && lane == 0) advance_launch_counter(a.ctr, gridDim.x * gridDim.y);
-}
-
-template <int N>
-static cudaError_t launch_quad_cluster_n(int map, bool two_d, cudaStream_t st, const KernelArgs &args)
-{
-    void (*k)(const KernelArgs);
-    int gx = (args.nx + 63) / 64, gy = args.ny;
-    switch (map) {
-    case kMapRow: k = two_d ? rlbm_quad_cluster_kernel<N, kMapRow, true> : rlbm_quad_cluster_kernel<N, kMapRow, false>; break;
-    case kMapCol:
-        k = rlbm_quad_cluster_kernel<N, kMapCol, true>;
-        gx = (args.nx + 31) / 32;
-        gy = (args.ny + 1) / 2;
-        break;
-    case kMapSplit: k = rlbm_quad_cluster_kernel<N, kMapSplit, false>; break;
-    default: return cudaErrorInvalidValue;
-    }
-    KernelArgs a = args;
-    a.cluster = quad_cluster_size(N);
-    const size_t smem = quad_cluster_smem(N, a.K);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(gx * a.cluster, gy);
-    cfg.blockDim = dim3(32, kQuadClusterWarps);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = a.cluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, a);
 }
 
 template <class St, int N, int PP, bool QUANT>

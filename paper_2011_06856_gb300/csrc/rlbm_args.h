@@ -72,7 +72,9 @@ struct KernelArgs {
     float2 rq[64], shellq[8];
     double rqd[64];      // the projection weights in FP64 (FP64 storage)
     float beta_f;        // stored-unit offset (FP32)
-    int cluster;         // CTAs per cluster of the many-angle quadrant kernel
+    float *split;        // many-angle quadrant kernel (rlbm_quad_split.cuh): ring of tiles' sums and coefficients,
+    unsigned *split_sync; // ticket, CTAs done, epoch, abort, then one counter per tile;
+    int split_cs, split_lag, split_ring; // CTAs per shell, tiles between a tile's two passes, tiles in the ring
     const int2 *shifts;  // npop: integer stencil vectors of the on-lattice rule (else NULL)
     double *qeta;        // quantum statistics: per site, eta = ln z of the last solve (the next
                          // step's Newton start; NaN: none yet), else NULL
@@ -147,15 +149,13 @@ __host__ __device__ constexpr size_t pair_smem_total(int N, int G, bool bulk, in
            (elem_bytes == 4 && pair_split(N, G) ? size_t(split_rows(N)) * kPairSites * 4 : 0);
 }
 
-// Many-angle quadrant kernel (rlbm_quad_cluster_kernel): CTAs per cluster, two per shell
-// (6 or 8, the portable size), warps per CTA, and dynamic shared memory: the angular sums of
-// the cluster's CTAs and of this CTA's warps, the per-site rows, 1 KB per quad.
-__host__ __device__ constexpr int quad_cluster_size(int N) { return 2 * (N + 1); }
-constexpr int kQuadClusterWarps = 10;
-__host__ __device__ constexpr size_t quad_cluster_smem(int N, int K)
+// Many-angle quadrant kernel (rlbm_quad_split.cuh): warps and resident CTAs per SM, and the
+// floats of a tile in the ring: the angular sums of its (N + 1) cs CTAs, the shells'
+// coefficients, U^a / tau.
+constexpr int kSplitWarps = 4, kSplitCtasPerSm = 5, kSplitSyncWords = 4;
+__host__ __device__ constexpr int split_tile_floats(int N, int cs)
 {
-    return size_t(5 * quad_cluster_size(N) + 5 * kQuadClusterWarps + pair_site_rows(N)) * kPairSites * 4 +
-           size_t((K / 4 + 1) / 2) * 1024;
+    return ((N + 1) * (5 * cs + 2 * N + 1) + 3) * kPairSites;
 }
 
 // Arguments of the persistent TMA-staged step kernel.
@@ -274,27 +274,20 @@ RLBM_DECLARE_QUAD(bf16)
 #undef RLBM_DECLARE_QUAD
 cudaError_t launch_quad_f64_n2(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
 cudaError_t launch_quad_f64_n3(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
-// many angles (FP32 storage): clusters of CTAs
-cudaError_t launch_quad_cluster_f32_n2(int map, bool two_d, cudaStream_t st, const KernelArgs &a);
-cudaError_t launch_quad_cluster_f32_n3(int map, bool two_d, cudaStream_t st, const KernelArgs &a);
-inline cudaError_t launch_quad_cluster_f32(int N, int map, bool two_d, cudaStream_t st, const KernelArgs &a)
-{
-    if (N == 2) return launch_quad_cluster_f32_n2(map, two_d, st, a);
-    if (N == 3) return launch_quad_cluster_f32_n3(map, two_d, st, a);
-    return cudaErrorInvalidValue;
-}
-// several population groups per warp (FP32 storage)
-cudaError_t launch_pair_groups_f32_n2(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                      const KernelArgs &a);
-cudaError_t launch_pair_groups_f32_n3(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                      const KernelArgs &a);
-inline cudaError_t launch_pair_groups_f32(int N, int PP, bool two_d, dim3 grid, dim3 block, size_t smem,
-                                          cudaStream_t st, const KernelArgs &a)
-{
-    if (N == 2) return launch_pair_groups_f32_n2(PP, two_d, grid, block, smem, st, a);
-    if (N == 3) return launch_pair_groups_f32_n3(PP, two_d, grid, block, smem, st, a);
-    return cudaErrorInvalidValue;
-}
+// many angles: two passes over the tiles in one launch
+#define RLBM_DECLARE_SPLIT(name)                                                                         \
+    cudaError_t launch_split_##name##_n2(int map, bool two_d, cudaStream_t st, const KernelArgs &a);     \
+    cudaError_t launch_split_##name##_n3(int map, bool two_d, cudaStream_t st, const KernelArgs &a);     \
+    inline cudaError_t launch_split_##name(int N, int map, bool two_d, cudaStream_t st, const KernelArgs &a) \
+    {                                                                                                    \
+        if (N == 2) return launch_split_##name##_n2(map, two_d, st, a);                                  \
+        if (N == 3) return launch_split_##name##_n3(map, two_d, st, a);                                  \
+        return cudaErrorInvalidValue;                                                                    \
+    }
+RLBM_DECLARE_SPLIT(f32)
+RLBM_DECLARE_SPLIT(f16)
+RLBM_DECLARE_SPLIT(bf16)
+#undef RLBM_DECLARE_SPLIT
 
 // Offsets of PairTmaSmem, formed once on the host (the kernel's warps would each repeat
 // about 60 integer instructions).

@@ -267,6 +267,7 @@ struct rlbm {
     int P = 0, Gs = 0, G = 0;
     int R = 1; // groups of P populations per warp (K beyond one group per warp)
     int stat = 0;       // equilibrium statistic: 0 Maxwell-Juttner, +1 Fermi-Dirac, -1 Bose-Einstein
+    void *d_split = nullptr;  // many angles: counters and ring of the two-pass kernel
     double *d_qeta = nullptr; // quantum statistics: per-site eta of the last solve (Newton warm start)
     double gdeg = 1.0;  // normalisation g of the quantum statistics
     bool site_fp64 = false;
@@ -693,6 +694,72 @@ bool quad_possible(const rlbm_t *h, int P)
            group_tiling(h->N, h->K, P, gs, ng) && ng == 1;
 }
 
+// Many angles: the two-pass quadrant kernel (rlbm_quad_split.cuh) where one CTA cannot hold
+// a tile's populations in registers, and for tilings that the quadrant kernel has no
+// instance of.  There the per-tile kernel is the alternative.  256^2, FP32, N = 2, us per
+// step, per-tile against two passes: ragged tilings (P not dividing K) N = 3, K = 100 292 to
+// 139, K = 84 240 to 129; P = 48 and K = 240 247 to 183.  Fewer than 128 angles in whole
+// warps stay with the per-tile kernel, whose CTAs hold them all (255 x 129, K = 96, P = 48:
+// 59 us, two passes 72), and so do 16-bit grids too small to fill the GPU, whose per-site
+// part is short (999 x 1, N = 3, K = 120: 19.4 us, two passes 21.3).
+constexpr int kSplitMinRaggedK = 64, kSplitMinK = 128, kSplitMinSites16 = 8192;
+bool split_wanted(const rlbm_t *h)
+{
+    return h->prec != RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && !h->stat && h->K % 4 == 0 &&
+           h->K >= (h->K % h->P ? kSplitMinRaggedK : kSplitMinK) && !quad_possible(h, h->P) &&
+           (storage_size(h->prec) > 2 || (long long)h->grid.nx * h->grid.ny >= kSplitMinSites16);
+}
+
+// Its ring and counters for the handle's present tiling (the stream is idle: creation and
+// retile).  A tile's two passes lie as many tiles apart as run at a time; the ring is three
+// times that.  Without memory the handle runs the per-tile kernel.
+void setup_split(rlbm_t *h)
+{
+    if (h->d_split) cudaFree(h->d_split);
+    h->d_split = nullptr;
+    if (!split_wanted(h)) return;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return;
+    const int resident = sms * rlbmk::kSplitCtasPerSm;
+    const long long tiles = std::max((h->grid.nx + 63ll) / 64 * h->grid.ny, (h->grid.nx + 31ll) / 32 * ((h->grid.ny + 1ll) / 2));
+    // one CTA per shell of a tile (a CTA's start and end cost as much as a few quads per
+    // warp: 256^2, N = 3, K = 600, one, two, four per shell 487, 514, 602 us); more only
+    // while the tiles do not fill the GPU, of at least two quads per warp
+    int cs = 1;
+    while (2 * cs * (h->N + 1) <= 16 && tiles * (h->N + 1) * cs < resident && h->K / 4 >= 2 * cs * 2 * rlbmk::kSplitWarps) cs *= 2;
+    const int parts = cs * (h->N + 1), lag = (resident + parts - 1) / parts, ring = 3 * lag;
+    const size_t sync = (size_t(rlbmk::kSplitSyncWords + tiles) * 4 + 255) / 256 * 256;
+    const size_t bytes = sync + size_t(ring) * rlbmk::split_tile_floats(h->N, cs) * 4;
+    if (2ll * parts * tiles > 0x7fffffffll || cudaMalloc(&h->d_split, bytes) != cudaSuccess ||
+        cudaMemsetAsync(h->d_split, 0, sync, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        if (h->d_split) cudaFree(h->d_split);
+        h->d_split = nullptr;
+        return;
+    }
+    h->base.split_sync = reinterpret_cast<unsigned *>(h->d_split);
+    h->base.split = reinterpret_cast<float *>(static_cast<unsigned char *>(h->d_split) + sync);
+    h->base.split_cs = cs;
+    h->base.split_lag = lag;
+    h->base.split_ring = ring;
+}
+
+cudaError_t launch_split(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
+{
+    const bool two_d = h->grid.ny > 1;
+    cudaError_t e;
+    switch (h->prec) {
+    case RLBM_FP32: e = rlbmk::launch_split_f32(h->N, map, two_d, h->stream, a); break;
+    case RLBM_FP16_DEV:
+    case RLBM_FP16_NORM: e = rlbmk::launch_split_f16(h->N, map, two_d, h->stream, a); break;
+    default: e = rlbmk::launch_split_bf16(h->N, map, two_d, h->stream, a); break;
+    }
+    if (e == cudaSuccess) ++h->launches;
+    return e;
+}
+
 // FP64 storage: the same conditions (P up to 32: the populations are kept in registers).
 bool quad64_possible(const rlbm_t *h)
 {
@@ -734,17 +801,12 @@ cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
 cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
     if (!h->pair_bulk && h->R == 1) return launch_quad(h, rlbmk::kMapRow, a);
+    if (h->d_split) return launch_split(h, rlbmk::kMapRow, a);
     const dim3 grid((h->grid.nx + rlbmk::kPairSites - 1) / rlbmk::kPairSites, h->grid.ny);
     const dim3 block(32, h->G);
-    // the population-groups kernel has no bulk staging
     const bool two_d = h->grid.ny > 1;
-    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, h->R == 1, int(storage_size(h->prec)), two_d);
+    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, true, int(storage_size(h->prec)), two_d);
     cudaError_t e;
-    if (h->R > 1) { // several population groups per warp (FP32 storage: pair_possible)
-        e = rlbmk::launch_pair_groups_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a);
-        if (e == cudaSuccess) ++h->launches;
-        return e;
-    }
     switch (h->prec) {
     case RLBM_FP32: e = rlbmk::launch_pair_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a); break;
     case RLBM_FP16_DEV:
@@ -825,6 +887,7 @@ cudaError_t launch_step(rlbm_t *h, int from)
     }
     const int map = h->grid.ny > 1 ? rlbmk::kMapCol : rlbmk::kMapSplit; // for any nx
     if (quad_possible(h, h->P)) return launch_quad(h, map, a);
+    if (h->d_split) return launch_split(h, map, a);
     if (quad64_possible(h)) return launch_quad64(h, a);
     return launch(h, rlbmk::MODE_STEP, a);
 }
@@ -1089,6 +1152,8 @@ rlbm_status retile(rlbm_t *h, int P, int kind)
     if (st) return st;
     st = setup_tma(h);
     if (st) return st;
+    setup_split(h);
+    if (h->use_pair && h->R > 1 && !h->d_split) h->use_pair = false; // no memory for it: the per-tile kernel
     h->use_pair_tma = false;
     if (h->use_pair && kind == 4) {
         st = setup_pair_tma(h);
@@ -1235,6 +1300,7 @@ static rlbm_status create_impl(rlbm_t **out, rlbm_grid grid, int order_N, int an
     }
     if (st == RLBM_OK) st = build_tables(h);
     if (st == RLBM_OK) st = setup_tma(h);
+    if (st == RLBM_OK) setup_split(h);
     if (st != RLBM_OK) {
         g_create_error = h->err;
         rlbm_destroy(h);
@@ -1319,6 +1385,7 @@ void rlbm_destroy(rlbm_t *h)
     if (h->d_tabs) cudaFree(h->d_tabs);
     if (h->d_status) cudaFree(h->d_status);
     if (h->d_qeta) cudaFree(h->d_qeta);
+    if (h->d_split) cudaFree(h->d_split);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete[] h->tma;
     delete[] h->ptma;

@@ -113,3 +113,47 @@ def test_unphysical_cell_is_reported_only_inside_the_grid():
         sim.step(1)
         with pytest.raises(R.Unphysical):
             sim.sync()
+
+
+# Many angles: two passes in one launch (csrc/rlbm_quad_split.cuh).  K / 4 even and odd, fewer
+# quads per CTA than warps, more; each way a lane's two sites lie; P is a tiling that leaves K
+# to the two passes; the widest grid has more tiles than the ring has places.
+@pytest.mark.parametrize("nx,ny,bcx,bcy", [(1, 1, PER, PER), (33, 3, OUT, OUT), (63, 1, OUT, PER), (66, 2, PER, OUT),
+                                           (130, 1, PER, PER)])
+@pytest.mark.parametrize("N,K,P", [(2, 100, 64), (3, 120, 48), (3, 120, 64), (2, 300, 64), (3, 288, 12), (2, 600, 24)])
+def test_fp32_many_angles(nx, ny, bcx, bcy, N, K, P):
+    pair = nx % 2 == 0 and K % P == 0 and P <= 32
+    for kind in ("per-tile", "pair") if pair else ("per-tile",):
+        f, m, ref, mac = run_both(nx, ny, N, K, 2.5, "fp32", bcx, bcy, P, kind, 4)
+        assert relerr(f, ref) < FP32_TOL and relerr(m[:2], mac[:2]) < FP32_TOL, kind
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16n"])
+def test_many_angles_more_tiles_than_ring_places(precision):
+    nx, ny, N, K = 513, 192, 2, 68
+    fl = W.random_fields(nx, ny, seed=4)
+    mom = {}
+    for p in (precision, "fp64"):
+        with R.Simulation(nx, ny, N, K, 2.5, p, OUT, PER) as sim:
+            sim.set_tiling(48, "per-tile")
+            sim.init_fields(fl)
+            sim.step(2)
+            sim.sync()
+            mom[p] = sim.moments()
+    assert relerr(mom[precision][:2], mom["fp64"][:2]) < (FP32_TOL if precision == "fp32" else 2 * 2.0 ** -10)
+
+
+def test_many_angles_report_an_unphysical_cell():
+    nx, ny, N, K = 33, 3, 3, 288
+    q = O.Quadrature(N, K)
+    fl = W.random_fields(nx, ny, seed=8)
+    with R.Simulation(nx, ny, N, K, 3.0, "fp32", OUT, OUT) as sim:
+        sim.init_fields(fl)
+        sim.step(2)
+        sim.sync()
+        f = q.init(fl.n, fl.T, fl.bx, fl.by).astype(np.float32)
+        f[:, ny - 1, nx - 1] *= -1.0
+        sim.set_populations(f)
+        sim.step(1)
+        with pytest.raises(R.Unphysical):
+            sim.sync()

@@ -386,28 +386,31 @@ __global__ void __launch_bounds__(128) apply_kernel(Net net, CoarseTab q, float 
 
 // ---------------------------------------------------------------- tensor-core apply
 // The fused correction with the three layers on BF16 tensor cores
-// (mma.sync.m16n8k16, FP32 accumulation), specialised for the coarse rule
-// (N, K).  A CTA of TC_WARPS warps works on tiles of 16 TC_WARPS sites; the
-// populations of the next tile stream into shared memory (cp.async, double
-// buffered) while the current one is processed.
+// (mma.sync.m16n8k16, FP32 accumulation), specialised for the coarse rule (N, K).
+//
+// A warp takes 16 sites at a time and needs nobody else: no CTA barriers, so that the
+// sixteen warps of an SM run through loads, arithmetic, products and stores at different
+// times.  (Tiles of 192 sites through shared memory, copied a tile ahead and processed in
+// step by twelve warps between CTA barriers, took 300 us on 1024^2 sites, K = 24, N = 2, at
+// 0.4 instructions a cycle and scheduler; the populations' one read and one write take 89.)
 //
 // * Conservation folded into the last layer.  With d = n0 W y (W = diag w) the
 //   projection d - W C^T A^-1 C d equals n0 W Q y, Q = I - C^T A^-1 C W, a
 //   constant matrix (C rows p^0, p^0 p^0, p^0 p^x, p^0 p^y; A = C W C^T).  So
-//   y' = Q y = h2 (W3 Q^T) + Q b3: each CTA forms W3' = W3 - (W3 V^T) U^T with
-//   V = C W and U = C^T A^-1 (FP32) and keeps it as a BF16 pair hi + lo
-//   (relative error 2^-17), so that C W y' vanishes to FP32 rounding.  The
-//   update is then f += n0 w_i y'_i.
-// * Features.  Warp w owns sites 16w..16w+15 of the tile; lane (site, half)
-//   sums half of every shell's angles (per-shell angular sums S0, Sc, Ss,
-//   Scc, Scs, Sss folded with p_r, p_r^2), the halves are joined by a shuffle,
-//   and the lane writes its populations / (w_i n0) as BF16 pairs into the
-//   warp's input row.
-// * Layers: [16 x K] x [K x N] products, fragments by ldmatrix from
-//   transposed, padded BF16 weights; GELU between them (gelu_as below).
-constexpr int TC_WARPS = 12;
-constexpr int TC_SITES = 16 * TC_WARPS; // sites per CTA tile
-constexpr int LDF = TC_SITES + 4;       // population-row stride of the tile (bank spread)
+//   y' = Q y = h2 (W3 Q^T) + Q b3: W3' = W3 - (W3 V^T) U^T with V = C W and U = C^T A^-1
+//   (FP32) is kept as a BF16 pair hi + lo (relative error 2^-17), so that C W y' vanishes to
+//   FP32 rounding.  The update is then f += n0 w_i y'_i.  The weights are laid out for the
+//   kernel's shared memory whenever they change (fold_kernel); each CTA only copies them.
+// * Features.  Lane (site, half) loads half of every shell's angles into registers, sums
+//   them (per-shell angular sums S0, Sc, Ss, Scc, Scs, Sss folded with p_r, p_r^2), the
+//   halves are joined by a shuffle, and the lane writes its populations / (w_i n0) as BF16
+//   pairs into the warp's input row.
+// * Layers: [16 x K] x [K x N] products, weight fragments by ldmatrix from transposed,
+//   padded BF16 weights; GELU between them (gelu2 below).  The accumulators of one layer
+//   have the layout of the next layer's left operand: the hidden layers stay in registers.
+// * Update: y' passes through the warp's shared memory to the lane that holds the site's
+//   populations.
+constexpr int TC_WARPS = 16;
 constexpr int SH = 72;                  // row stride of hidden tiles and of W2^T, W3'^T
 
 __device__ __forceinline__ void mma_bf16(float *d, unsigned a0, unsigned a1, unsigned a2, unsigned a3,
@@ -447,42 +450,25 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
 // GELU(x) = x Phi(x) = x (1 + erf(x / sqrt 2)) / 2 with erf from Abramowitz &
 // Stegun 7.1.26 (Hastings' rational approximation, |error| <= 1.5e-7):
 // erf(z) = 1 - t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2), t = 1 / (1 + p z),
-// z >= 0, extended to z < 0 by symmetry.  The layers' inputs are BF16, so
-// this accuracy is far below their rounding.
-__device__ __forceinline__ float gelu_as(float x)
-{
-    const float z = fabsf(x) * 0.70710678118654752f;
-    float t;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, z, 1.0f)));
-    float q = fmaf(1.061405429f, t, -1.453152027f);
-    q = fmaf(q, t, 1.421413741f);
-    q = fmaf(q, t, -0.284496736f);
-    q = fmaf(q, t, 0.254829592f);
-    q *= t;
-    float e; // exp(-z^2)
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-1.4426950408889634f * z * z));
-    const float h = 0.5f * q * e;                          // (1 - erf(z)) / 2
-    return x * (x >= 0.f ? 1.f - h : h);
-}
-
-// GELU of two values with packed f32x2 arithmetic (same formula as gelu_as)
+// z = |x| / sqrt 2, extended to x < 0 by symmetry.  The layers' inputs are BF16, so
+// this accuracy is far below their rounding.  Two values with packed arithmetic; the factors
+// 1 / sqrt 2 and 1 / 2 are in the constants.
 __device__ __forceinline__ float2 gelu2(float2 x)
 {
-    const float2 z = make_float2(fabsf(x.x) * 0.70710678118654752f, fabsf(x.y) * 0.70710678118654752f);
-    const float2 den = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), z, make_float2(1.f, 1.f));
-    float2 t;
+    constexpr float P = 0.3275911f * 0.70710678118654752f;
+    const float2 den = __ffma2_rn(make_float2(P, P), make_float2(fabsf(x.x), fabsf(x.y)), make_float2(1.f, 1.f));
+    const float2 a = __fmul2_rn(__fmul2_rn(x, x), make_float2(-0.72134752044448170f, -0.72134752044448170f));
+    float2 t, e; // e = exp(-x^2 / 2)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(den.x));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(den.y));
-    float2 q = __ffma2_rn(make_float2(1.061405429f, 1.061405429f), t, make_float2(-1.453152027f, -1.453152027f));
-    q = __ffma2_rn(q, t, make_float2(1.421413741f, 1.421413741f));
-    q = __ffma2_rn(q, t, make_float2(-0.284496736f, -0.284496736f));
-    q = __ffma2_rn(q, t, make_float2(0.254829592f, 0.254829592f));
-    q = __fmul2_rn(q, t);
-    const float2 a = __fmul2_rn(__fmul2_rn(z, z), make_float2(-1.4426950408889634f, -1.4426950408889634f));
-    float2 e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(a.x));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(a.y));
-    const float2 xh = __fmul2_rn(x, __fmul2_rn(__fmul2_rn(q, e), make_float2(0.5f, 0.5f))); // x (1 - erf(z)) / 2
+    float2 q = __ffma2_rn(make_float2(0.5f * 1.061405429f, 0.5f * 1.061405429f), t,
+                          make_float2(0.5f * -1.453152027f, 0.5f * -1.453152027f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * 1.421413741f, 0.5f * 1.421413741f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * -0.284496736f, 0.5f * -0.284496736f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * 0.254829592f, 0.5f * 0.254829592f));
+    const float2 xh = __fmul2_rn(x, __fmul2_rn(__fmul2_rn(q, t), e)); // x (1 - erf(z)) / 2
     return make_float2(x.x >= 0.f ? x.x - xh.x : xh.x, x.y >= 0.f ? x.y - xh.y : xh.y);
 }
 
@@ -535,42 +521,38 @@ __device__ __forceinline__ void gelu_rows(float (*acc)[4], __nv_bfloat16 *h, int
     }
 }
 
-// Populations of the tile at site0 into the shared tile (rows of LDF floats);
-// sites >= S read as zero.  VEC = 4: 16-byte copies (S % 4 == 0, f 16-byte
-// aligned); VEC = 1: 4-byte copies.
-template <int VEC>
-__device__ __forceinline__ void load_tile(float *tile, const float *f, long long S, long long site0, int npop)
+// The next layer's left operand from a layer's accumulators: GELU, rounded to BF16.
+__device__ __forceinline__ void gelu_frags(const float (*acc)[4], unsigned (*h)[4])
 {
-    constexpr int CH = TC_SITES / VEC;
-    for (int e = threadIdx.x; e < npop * CH; e += blockDim.x) {
-        const int i = e / CH, c = e % CH;
-        const long long site = site0 + c * VEC;
-        const bool ok = site < S;
-        const float *src = ok ? f + (long long)i * S + site : f;
-        const unsigned dst = smem_addr(tile + i * LDF + c * VEC);
-        if (VEC == 4)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0)
-                         : "memory");
-        else
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0)
-                         : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { // rows g, g + 8 at columns 2t, then at 2t + 8
+            const float *z = acc[2 * ks + (u >> 1)] + 2 * (u & 1);
+            const float2 v = gelu2(make_float2(z[0], z[1]));
+            h[ks][u] = pack_bf16(v.x, v.y);
+        }
 }
 
-template <int VEC>
-__device__ __forceinline__ void store_tile(const float *tile, float *f, long long S, long long site0, int npop)
+// acc[nt][4] += H[16 x 64] (fragments) x Bt[8 NT x 64]^T (row stride SH)
+template <int NT>
+__device__ __forceinline__ void frag_gemm(const unsigned (*h)[4], const __nv_bfloat16 *Bt, float (*acc)[4], int lane)
 {
-    constexpr int CH = TC_SITES / VEC;
-    for (int e = threadIdx.x; e < npop * CH; e += blockDim.x) {
-        const int i = e / CH, c = e % CH;
-        const long long site = site0 + c * VEC;
-        if (site >= S) continue;
-        if (VEC == 4)
-            *reinterpret_cast<float4 *>(f + (long long)i * S + site) =
-                *reinterpret_cast<const float4 *>(tile + i * LDF + c * 4);
-        else
-            f[(long long)i * S + site] = tile[i * LDF + c];
+    const int mi = lane >> 3, r8 = lane & 7;
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+#pragma unroll
+        for (int np = 0; np < NT / 2; ++np) {
+            unsigned b0, b1, b2, b3;
+            ldsm_x4(Bt + (np * 16 + (mi >> 1) * 8 + r8) * SH + ks * 16 + (mi & 1) * 8, b0, b1, b2, b3);
+            mma_bf16(acc[2 * np], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b0, b1);
+            mma_bf16(acc[2 * np + 1], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b2, b3);
+        }
+        if (NT & 1) {
+            unsigned b0, b1;
+            ldsm_x2(Bt + ((NT - 1) * 8 + r8) * SH + ks * 16 + (mi & 1) * 8, b0, b1);
+            mma_bf16(acc[NT - 1], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b0, b1);
+        }
     }
 }
 
@@ -581,116 +563,122 @@ struct TcGeom {
     static constexpr int KS1 = (F + 15) / 16; // k-steps of layer 1
     static constexpr int SX = 16 * KS1 + 8;   // input row stride: odd number of 16-byte units
     static constexpr int NT3 = NPOP / 8;      // n-tiles of layer 3
-    // shared memory carve-up, bytes
+    static constexpr int LY = NPOP + 2;       // row stride of y': 64-bit reads of 16 rows without bank conflicts
+    // the prepared weights and tables (fold_kernel), copied to the start of shared memory
     static constexpr size_t W1 = 0, W2 = W1 + size_t(64) * SX * 2, W3H = W2 + size_t(64) * SH * 2,
                             W3L = W3H + size_t(NPOP) * SH * 2, BIAS = W3L + size_t(NPOP) * SH * 2,
-                            TAB = BIAS + size_t(128 + NPOP) * 4,
-                            WV = TAB + size_t(4 * NPOP + 8) * 4, // cs (2 NPOP), invw, wq, p_r (<= 8)
-                            FT = (WV + 64 * 4 * 4 + 8 * 4 + 15) / 16 * 16,
-                            WARP = FT + size_t(2) * NPOP * LDF * 4, TOTAL = WARP + size_t(TC_WARPS) * 16 * SX * 2;
+                            TAB = BIAS + size_t(128 + NPOP) * 4, // b1 b2 b3' | v_x, v_y, 1 / w, w per population, p_r
+                            FOLD = (TAB + size_t(4 * NPOP + 8) * 4 + 15) / 16 * 16,
+                            XA = size_t(16) * SX * 2, YS = size_t(16) * LY * 4, // a warp's input rows, y'
+                            WARP = ((XA > YS ? XA : YS) + 15) / 16 * 16, TOTAL = FOLD + TC_WARPS * WARP;
 };
+constexpr size_t kFoldMaxBytes = 64 * 1024;
 
-template <int N, int K, int VEC>
-__global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(Net net, CoarseTab q, float *__restrict__ f,
-                                                                    long long S, float kn)
+// The BF16 weights, the folded last layer and the tables in the layout of apply_tc_kernel's
+// shared memory; one thread per element, the projections (W3 V^T)[64][4], (V b3)[4] once per CTA.
+template <int N, int K>
+__global__ void __launch_bounds__(256) fold_kernel(Net net, CoarseTab q, unsigned char *fold)
 {
     using Gm = TcGeom<N, K>;
-    constexpr int NPOP = Gm::NPOP, F = Gm::F, SX = Gm::SX, KH = K / 2;
-    static_assert(K % 4 == 0 && NPOP % 8 == 0 && NPOP <= 2 * 64, "tile geometry");
-    extern __shared__ __align__(16) unsigned char sm[];
-    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W1);  // [64][SX]
-    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W2);  // [64][SH]
-    __nv_bfloat16 *w3h = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W3H); // [NPOP][SH]
-    __nv_bfloat16 *w3l = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W3L); // [NPOP][SH]
-    float *bias = reinterpret_cast<float *>(sm + Gm::BIAS);               // b1[64] b2[64] b3'[NPOP]
-    float *cvec = reinterpret_cast<float *>(sm + Gm::TAB);                // v_x per population
-    float *svec = cvec + NPOP;                                            // v_y per population
-    float *invw = svec + NPOP;
-    float *wq = invw + NPOP;
-    float *pr = wq + NPOP;                                                // p_r per shell
-    float *wv = reinterpret_cast<float *>(sm + Gm::WV);                   // (W3 V^T)[64][4], V b3 [4]
-    float *ftile = reinterpret_cast<float *>(sm + Gm::FT);                // [2][NPOP][LDF]
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    __nv_bfloat16 *xa = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::WARP) + size_t(wid) * 16 * SX;
-    const long long ntile = (S + TC_SITES - 1) / TC_SITES;
-    long long tile = blockIdx.x;
-    if (tile < ntile) load_tile<VEC>(ftile, f, S, tile * TC_SITES, NPOP);
-
-    // ---- per-CTA setup: weights, tables, the folded last layer
-    for (int e = tid; e < 64 * SX; e += blockDim.x) {
-        const int n = e / SX, k = e % SX;
-        w1t[e] = (k < F) ? net.W1[k * H + n] : __float2bfloat16_rn(0.f);
-    }
-    for (int e = tid; e < 64 * SH; e += blockDim.x) {
-        const int n = e / SH, k = e % SH;
-        w2t[e] = (k < H) ? net.W2[k * H + n] : __float2bfloat16_rn(0.f);
-    }
-    for (int e = tid; e < 64; e += blockDim.x) { bias[e] = net.b1[e]; bias[64 + e] = net.b2[e]; }
-    for (int e = tid; e < NPOP; e += blockDim.x) {
-        cvec[e] = q.c[e];
-        svec[e] = q.s[e];
-        invw[e] = 1.f / q.w[e];
-        wq[e] = q.w[e];
-    }
-    for (int e = tid; e <= N; e += blockDim.x) pr[e] = q.p0[e * K];
+    constexpr int NPOP = Gm::NPOP, F = Gm::F, SX = Gm::SX;
+    static_assert(Gm::FOLD <= kFoldMaxBytes, "fold buffer");
+    __shared__ float cm[4][NPOP], wv[65 * 4];
+    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W1);
+    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W2);
+    __nv_bfloat16 *w3h = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W3H);
+    __nv_bfloat16 *w3l = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W3L);
+    float *bias = reinterpret_cast<float *>(fold + Gm::BIAS), *tab = reinterpret_cast<float *>(fold + Gm::TAB);
     // C[a][j] for a = 0..3: p, p^2, p^2 c, p^2 s
-    auto Cm = [&](int a0, int j) {
+    for (int j = threadIdx.x; j < NPOP; j += blockDim.x) {
         const float p = q.p0[j];
-        return a0 == 0 ? p : a0 == 1 ? p * p : a0 == 2 ? p * p * q.c[j] : p * p * q.s[j];
-    };
-    // (W3 V^T)[k][a] = sum_j W3[k][j] C[a][j] w_j, and (V b3)[a]
-    for (int e = tid; e < 64 * 4 + 4; e += blockDim.x) {
+        cm[0][j] = p;
+        cm[1][j] = p * p;
+        cm[2][j] = p * p * q.c[j];
+        cm[3][j] = p * p * q.s[j];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 65 * 4; e += blockDim.x) {
+        const int k = e >> 2, a = e & 3;
         float acc = 0.f;
-        if (e < 256) {
-            const int k = e >> 2, a0 = e & 3;
-            for (int j = 0; j < NPOP; ++j) acc += __bfloat162float(net.W3[k * NPOP + j]) * Cm(a0, j) * q.w[j];
-        } else {
-            const int a0 = e - 256;
-            for (int j = 0; j < NPOP; ++j) acc += net.b3[j] * Cm(a0, j) * q.w[j];
-        }
+#pragma unroll 8
+        for (int j = 0; j < NPOP; ++j) acc += (k < 64 ? __bfloat162float(net.W3[k * NPOP + j]) : net.b3[j]) * cm[a][j] * q.w[j];
         wv[e] = acc;
     }
     __syncthreads();
-    // W3'[k][i] = W3[k][i] - sum_a (W3 V^T)[k][a] U[i][a], U = C^T A^-1; b3' likewise
-    for (int e = tid; e < NPOP * SH; e += blockDim.x) {
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
+    for (int e = t0; e < 64 * SX; e += nt) w1t[e] = e % SX < F ? net.W1[(e % SX) * H + e / SX] : zero;
+    for (int e = t0; e < 64 * SH; e += nt) w2t[e] = e % SH < H ? net.W2[(e % SH) * H + e / SH] : zero;
+    // W3'[k][i] = W3[k][i] - sum_a (W3 V^T)[k][a] U[i][a], U = C^T A^-1; b3' likewise (k = 64)
+    for (int e = t0; e < NPOP * SH; e += nt) {
         const int i = e / SH, k = e % SH;
-        float u[4];
+        float v = 0.f;
+        if (k <= H) {
+            v = k < H ? __bfloat162float(net.W3[k * NPOP + i]) : net.b3[i];
+            float d = 0.f;
 #pragma unroll
-        for (int a0 = 0; a0 < 4; ++a0)
-            u[a0] = Cm(0, i) * q.Ainv[0 * 4 + a0] + Cm(1, i) * q.Ainv[1 * 4 + a0] + Cm(2, i) * q.Ainv[2 * 4 + a0] +
-                    Cm(3, i) * q.Ainv[3 * 4 + a0];
-        if (k < H) {
-            const float v = __bfloat162float(net.W3[k * NPOP + i]) -
-                            (wv[k * 4] * u[0] + wv[k * 4 + 1] * u[1] + wv[k * 4 + 2] * u[2] + wv[k * 4 + 3] * u[3]);
-            const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-            w3h[e] = hi;
-            w3l[e] = __float2bfloat16_rn(v - __bfloat162float(hi));
-        } else {
-            w3h[e] = __float2bfloat16_rn(0.f);
-            w3l[e] = __float2bfloat16_rn(0.f);
+            for (int a = 0; a < 4; ++a)
+                d += wv[k * 4 + a] * (cm[0][i] * q.Ainv[a] + cm[1][i] * q.Ainv[4 + a] + cm[2][i] * q.Ainv[8 + a] + cm[3][i] * q.Ainv[12 + a]);
+            v -= d;
         }
-        if (k == 0)
-            bias[128 + i] = net.b3[i] - (wv[256] * u[0] + wv[257] * u[1] + wv[258] * u[2] + wv[259] * u[3]);
+        if (k == H) bias[128 + i] = v;
+        const __nv_bfloat16 hi = __float2bfloat16_rn(k < H ? v : 0.f);
+        w3h[e] = hi;
+        w3l[e] = __float2bfloat16_rn(k < H ? v - __bfloat162float(hi) : 0.f);
     }
-    for (int e = lane; e < 16 * SX; e += 32) xa[e] = __float2bfloat16_rn(0.f);
+    for (int e = t0; e < 128; e += nt) bias[e] = e < 64 ? net.b1[e] : net.b2[e - 64];
+    for (int e = t0; e < NPOP; e += nt) {
+        tab[e] = q.c[e];
+        tab[NPOP + e] = q.s[e];
+        tab[2 * NPOP + e] = 1.f / q.w[e];
+        tab[3 * NPOP + e] = q.w[e];
+    }
+    for (int e = t0; e < 8; e += nt) tab[4 * NPOP + e] = e <= N ? q.p0[e * K] : 0.f;
+}
+
+template <int N, int K>
+__global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsigned char *__restrict__ fold, float *__restrict__ f,
+                                                                    long long S, float kn)
+{
+    using Gm = TcGeom<N, K>;
+    constexpr int NPOP = Gm::NPOP, F = Gm::F, SX = Gm::SX, KH = K / 2, LY = Gm::LY;
+    static_assert(K % 4 == 0 && NPOP % 8 == 0 && NPOP <= 2 * 64, "tile geometry");
+    extern __shared__ __align__(16) unsigned char sm[];
+    const __nv_bfloat16 *w1t = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W1);  // [64][SX]
+    const __nv_bfloat16 *w2t = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W2);  // [64][SH]
+    const __nv_bfloat16 *w3h = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W3H); // [NPOP][SH]
+    const __nv_bfloat16 *w3l = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W3L); // [NPOP][SH]
+    const float *bias = reinterpret_cast<const float *>(sm + Gm::BIAS);               // b1[64] b2[64] b3'[NPOP]
+    const float *cvec = reinterpret_cast<const float *>(sm + Gm::TAB);                // v_x per population
+    const float *svec = cvec + NPOP, *invw = svec + NPOP, *wq = invw + NPOP;
+    const float *pr = wq + NPOP;                                                      // p_r per shell
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int e = tid; e < int(Gm::FOLD / 16); e += TC_WARPS * 32)
+        reinterpret_cast<uint4 *>(sm)[e] = __ldg(reinterpret_cast<const uint4 *>(fold) + e);
     __syncthreads();
+    unsigned char *own = sm + Gm::FOLD + size_t(wid) * Gm::WARP;
+    __nv_bfloat16 *xa = reinterpret_cast<__nv_bfloat16 *>(own); // [16][SX], then
+    float *ys = reinterpret_cast<float *>(own);                 // [16][LY]
 
     const int g = lane >> 2, t = lane & 3;
     const int ls = lane & 15, half = lane >> 4;
-    for (int k = 0; tile < ntile; ++k, tile += gridDim.x) {
-        float *cur = ftile + (k & 1) * NPOP * LDF;
-        const long long site0 = tile * TC_SITES;
-        if (tile + gridDim.x < ntile)
-            load_tile<VEC>(ftile + ((k + 1) & 1) * NPOP * LDF, f, S, (tile + gridDim.x) * TC_SITES, NPOP);
-        else
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();
-        // ---- features of the warp's 16 sites: this lane takes angles [half K/2, (half+1) K/2) of every shell
-        const int col = wid * 16 + ls;
-        const bool valid = site0 + col < S;
-        // populations in pairs (i, i+1): the angular sums run on packed f32x2 operands
+    const long long ngroup = (S + 15) / 16, nwarp = (long long)gridDim.x * TC_WARPS;
+    // groups next to each other run at the same time: their rows share DRAM pages
+    for (long long group = (long long)blockIdx.x * TC_WARPS + wid; group < ngroup; group += nwarp) {
+        const long long site = group * 16 + ls;
+        const bool valid = site < S;
+        // ---- this lane takes angles [half K/2, (half+1) K/2) of every shell of its site
+        float *fs = f + (long long)(half * KH) * S + (valid ? site : 0);
         float2 v[N + 1][KH / 2];
+        {
+            const float *p = fs;
+#pragma unroll
+            for (int r = 0; r <= N; ++r) {
+#pragma unroll
+                for (int jj = 0; jj < KH / 2; ++jj, p += 2 * S) v[r][jj] = make_float2(p[0], p[S]);
+                p += (long long)(K - KH) * S;
+            }
+        }
         float m[9];
 #pragma unroll
         for (int a0 = 0; a0 < 9; ++a0) m[a0] = 0.f;
@@ -700,10 +688,9 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(Net net, Coa
 #pragma unroll
             for (int jj = 0; jj < KH; jj += 2) {
                 const int i = r * K + half * KH + jj;
-                const float2 x = make_float2(cur[i * LDF + col], cur[(i + 1) * LDF + col]);
+                const float2 x = v[r][jj / 2];
                 const float2 cp = *reinterpret_cast<const float2 *>(cvec + i);
                 const float2 sp = *reinterpret_cast<const float2 *>(svec + i);
-                v[r][jj / 2] = x;
                 const float2 cx = __fmul2_rn(cp, x), sx = __fmul2_rn(sp, x);
                 S0 = __fadd2_rn(S0, x); Sc = __fadd2_rn(Sc, cx); Ss = __fadd2_rn(Ss, sx);
                 Scc = __ffma2_rn(cp, cx, Scc); Scs = __ffma2_rn(cp, sx, Scs); Sss = __ffma2_rn(sp, sx, Sss);
@@ -718,6 +705,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(Net net, Coa
 #pragma unroll
         for (int a0 = 0; a0 < 9; ++a0) m[a0] += __shfl_xor_sync(0xffffffffu, m[a0], 16);
         const float n0 = m[0], inv = valid ? __frcp_rn(n0) : 0.f;
+        __syncwarp(); // y' of the previous group has been read
         __nv_bfloat16 *xr = xa + ls * SX;
         if (half == 0) {
 #pragma unroll
@@ -734,56 +722,67 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(Net net, Coa
                 const float2 sc2 = __fmul2_rn(__fmul2_rn(v[r][jj / 2], iw), make_float2(inv, inv));
                 *reinterpret_cast<unsigned *>(xr + 10 + i) = pack_bf16(sc2.x, sc2.y);
             }
-        // zero padding of layer 1's k range (the hidden tile of the previous tile overlaps it)
+        // zero padding of layer 1's k range (y' of the previous group overlaps it)
         constexpr int PADP = (16 * Gm::KS1 - F) / 2;
         for (int e = lane; e < 16 * PADP; e += 32)
             *reinterpret_cast<unsigned *>(xa + (e / PADP) * SX + F + 2 * (e % PADP)) = 0u;
         __syncwarp();
-        // ---- layer 1: [16 x 16 KS1] x [16 KS1 x 64]; the hidden tile reuses the input rows
+        // ---- layers 1, 2, 3 (folded projection, hi + lo)
         float acc[Gm::NT3 > 8 ? Gm::NT3 : 8][4];
+        unsigned h[4][4];
         bias_init(acc, bias, 8, lane);
         warp_gemm<Gm::KS1, 8>(xa, SX, w1t, SX, acc, lane);
-        __syncwarp();
-        gelu_rows(acc, xa, lane);
-        __syncwarp();
-        // ---- layer 2
+        gelu_frags(acc, h);
         bias_init(acc, bias + 64, 8, lane);
-        warp_gemm<4, 8>(xa, SH, w2t, SH, acc, lane);
-        __syncwarp();
-        gelu_rows(acc, xa, lane);
-        __syncwarp();
-        // ---- layer 3 with the folded projection (hi + lo)
+        frag_gemm<8>(h, w2t, acc, lane);
+        gelu_frags(acc, h);
         bias_init(acc, bias + 128, Gm::NT3, lane);
-        warp_gemm<4, Gm::NT3>(xa, SH, w3h, SH, acc, lane);
-        warp_gemm<4, Gm::NT3>(xa, SH, w3l, SH, acc, lane);
-        // ---- update: f_i += n0 w_i y'_i; rows g (u = 0, 1) and g + 8 (u = 2, 3)
-        const float na = __shfl_sync(0xffffffffu, n0, g), nb = __shfl_sync(0xffffffffu, n0, g + 8);
-        float *fa = cur + wid * 16 + g;
+        frag_gemm<Gm::NT3>(h, w3h, acc, lane);
+        frag_gemm<Gm::NT3>(h, w3l, acc, lane);
+        __syncwarp(); // every lane has read its input rows
 #pragma unroll
-        for (int nt = 0; nt < Gm::NT3; ++nt) {
+        for (int nt = 0; nt < Gm::NT3; ++nt) { // rows g (u = 0, 1) and g + 8 (u = 2, 3)
             const int c = nt * 8 + 2 * t;
-            const float2 w2 = *reinterpret_cast<const float2 *>(wq + c);
-            fa[c * LDF] = fmaf(na * w2.x, acc[nt][0], fa[c * LDF]);
-            fa[(c + 1) * LDF] = fmaf(na * w2.y, acc[nt][1], fa[(c + 1) * LDF]);
-            fa[c * LDF + 8] = fmaf(nb * w2.x, acc[nt][2], fa[c * LDF + 8]);
-            fa[(c + 1) * LDF + 8] = fmaf(nb * w2.y, acc[nt][3], fa[(c + 1) * LDF + 8]);
+            *reinterpret_cast<float2 *>(ys + g * LY + c) = make_float2(acc[nt][0], acc[nt][1]);
+            *reinterpret_cast<float2 *>(ys + (g + 8) * LY + c) = make_float2(acc[nt][2], acc[nt][3]);
         }
-        __syncthreads();
-        store_tile<VEC>(cur, f, S, site0, NPOP);
-        __syncthreads(); // the buffer is refilled by the next iteration's copy
+        __syncwarp();
+        // ---- update: f_i += n0 w_i y'_i
+        if (valid) {
+            float *p = fs;
+#pragma unroll
+            for (int r = 0; r <= N; ++r) {
+#pragma unroll
+                for (int jj = 0; jj < KH; jj += 2, p += 2 * S) {
+                    const int i = r * K + half * KH + jj;
+                    const float2 w2 = *reinterpret_cast<const float2 *>(wq + i);
+                    const float2 y = *reinterpret_cast<const float2 *>(ys + ls * LY + i);
+                    const float2 out = __ffma2_rn(__fmul2_rn(make_float2(n0, n0), w2), y, v[r][jj / 2]);
+                    p[0] = out.x;
+                    p[S] = out.y;
+                }
+                p += (long long)(K - KH) * S;
+            }
+        }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-using TcKernel = void (*)(Net, CoarseTab, float *, long long, float);
+using TcKernel = void (*)(const unsigned char *, float *, long long, float);
+using FoldKernel = void (*)(Net, CoarseTab, unsigned char *);
 
 // the specialisations: (N, K) with N_pop a multiple of 8 and at most 80 outputs
-template <int VEC>
 TcKernel tc_kernel(int N, int K, size_t *smem)
 {
-    if (N == 2 && K == 24) { *smem = TcGeom<2, 24>::TOTAL; return apply_tc_kernel<2, 24, VEC>; }
-    if (N == 2 && K == 16) { *smem = TcGeom<2, 16>::TOTAL; return apply_tc_kernel<2, 16, VEC>; }
-    if (N == 3 && K == 16) { *smem = TcGeom<3, 16>::TOTAL; return apply_tc_kernel<3, 16, VEC>; }
+    if (N == 2 && K == 24) { *smem = TcGeom<2, 24>::TOTAL; return apply_tc_kernel<2, 24>; }
+    if (N == 2 && K == 16) { *smem = TcGeom<2, 16>::TOTAL; return apply_tc_kernel<2, 16>; }
+    if (N == 3 && K == 16) { *smem = TcGeom<3, 16>::TOTAL; return apply_tc_kernel<3, 16>; }
+    return nullptr;
+}
+FoldKernel fold_kernel_of(int N, int K)
+{
+    if (N == 2 && K == 24) return fold_kernel<2, 24>;
+    if (N == 2 && K == 16) return fold_kernel<2, 16>;
+    if (N == 3 && K == 16) return fold_kernel<3, 16>;
     return nullptr;
 }
 
@@ -1072,6 +1071,7 @@ struct rlbm_closure {
     int *d_wmap = nullptr;          // BF16 weight -> master index
     float *d_tab = nullptr;         // p0 | c | s | w | Ainv
     float *d_loss = nullptr;
+    unsigned char *d_fold = nullptr; // weights and tables as apply_tc_kernel keeps them in shared memory
     int adam_t = 0;
     bool simt_apply = false;
     bool simt_train = false;
@@ -1143,13 +1143,9 @@ bool tc_attributes(const rlbm_closure *c)
     TrKernel tk = tr_kernel(c->N, c->K, &trsmem);
     if (tk && cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsmem) != cudaSuccess)
         return false;
-    for (int v = 0; v < 2; ++v) {
-        size_t smem = 0;
-        TcKernel k = v ? tc_kernel<4>(c->N, c->K, &smem) : tc_kernel<1>(c->N, c->K, &smem);
-        if (k && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return false;
-    }
-    return true;
+    size_t smem = 0;
+    TcKernel k = tc_kernel(c->N, c->K, &smem);
+    return !k || cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
 }
 
 rlbm_status refresh_bf16(rlbm_closure *c)
@@ -1157,6 +1153,10 @@ rlbm_status refresh_bf16(rlbm_closure *c)
     const int nw = c->F * H + H * H + H * c->O;
     to_bf16_kernel<<<(nw + 255) / 256, 256, 0, c->stream>>>(c->d_p, c->d_w, c->d_wmap, nw);
     CL_CUDA(c, cudaGetLastError());
+    if (FoldKernel k = fold_kernel_of(c->N, c->K)) { // in stream order, also under capture
+        k<<<16, 256, 0, c->stream>>>(net_of(c), tab_of(c), c->d_fold);
+        CL_CUDA(c, cudaGetLastError());
+    }
     return RLBM_OK;
 }
 
@@ -1257,7 +1257,8 @@ rlbm_status rlbm_closure_create(rlbm_closure_t **out, int order_N, int angles_K,
     if (cudaMalloc(&c->d_p, c->nparam * 4) != cudaSuccess || cudaMalloc(&c->d_g, c->nparam * 4) != cudaSuccess ||
         cudaMalloc(&c->d_m, c->nparam * 4) != cudaSuccess || cudaMalloc(&c->d_v, c->nparam * 4) != cudaSuccess ||
         cudaMalloc(&c->d_w, size_t(nw) * 2) != cudaSuccess || cudaMalloc(&c->d_wmap, size_t(nw) * 4) != cudaSuccess ||
-        cudaMalloc(&c->d_tab, tab.size() * 4) != cudaSuccess || cudaMalloc(&c->d_loss, 4) != cudaSuccess)
+        cudaMalloc(&c->d_tab, tab.size() * 4) != cudaSuccess || cudaMalloc(&c->d_loss, 4) != cudaSuccess ||
+        cudaMalloc(&c->d_fold, kFoldMaxBytes) != cudaSuccess)
         return bail(cfail(c, RLBM_ERR_OOM, "device allocation failed"));
     if (cudaMemcpyAsync(c->d_p, p.data(), c->nparam * 4, cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->d_m, 0, c->nparam * 4, c->stream) != cudaSuccess ||
@@ -1283,7 +1284,7 @@ void rlbm_closure_destroy(rlbm_closure_t *c)
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     cudaFree(c->d_p); cudaFree(c->d_g); cudaFree(c->d_m); cudaFree(c->d_v);
-    cudaFree(c->d_w); cudaFree(c->d_wmap); cudaFree(c->d_tab); cudaFree(c->d_loss);
+    cudaFree(c->d_w); cudaFree(c->d_wmap); cudaFree(c->d_tab); cudaFree(c->d_loss); cudaFree(c->d_fold);
     delete c;
 }
 
@@ -1468,16 +1469,15 @@ rlbm_status rlbm_closure_apply_buffer(rlbm_closure_t *c, float *d_f, long long s
 {
     if (!c || !d_f || sites < 1) return cfail(c, RLBM_ERR_ARG, "bad arguments");
     size_t smem = 0;
-    const bool vec = sites % 4 == 0 && reinterpret_cast<uintptr_t>(d_f) % 16 == 0;
-    TcKernel k = c->simt_apply ? nullptr : vec ? tc_kernel<4>(c->N, c->K, &smem) : tc_kernel<1>(c->N, c->K, &smem);
+    TcKernel k = c->simt_apply ? nullptr : tc_kernel(c->N, c->K, &smem);
     if (k) {
         // tensor-core path: a persistent grid of one CTA per SM
         int dev = 0, sms = 0;
         CL_CUDA(c, cudaGetDevice(&dev));
         CL_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const long long tiles = (sites + TC_SITES - 1) / TC_SITES;
+        const long long tiles = (sites + 16 * TC_WARPS - 1) / (16 * TC_WARPS);
         const int grid = int(std::min<long long>(sms, tiles));
-        k<<<grid, TC_WARPS * 32, smem, c->stream>>>(net_of(c), tab_of(c), d_f, sites, float(kn));
+        k<<<grid, TC_WARPS * 32, smem, c->stream>>>(c->d_fold, d_f, sites, float(kn));
         CL_CUDA(c, cudaGetLastError());
         return RLBM_OK;
     }

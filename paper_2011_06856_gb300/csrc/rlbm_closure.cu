@@ -508,19 +508,6 @@ __device__ __forceinline__ void bias_init(float (*acc)[4], const float *b, int n
     }
 }
 
-__device__ __forceinline__ void gelu_rows(float (*acc)[4], __nv_bfloat16 *h, int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int c = nt * 8 + t * 2;
-        const float2 a = gelu2(make_float2(acc[nt][0], acc[nt][1]));
-        const float2 b = gelu2(make_float2(acc[nt][2], acc[nt][3]));
-        *reinterpret_cast<unsigned *>(h + g * SH + c) = pack_bf16(a.x, a.y);
-        *reinterpret_cast<unsigned *>(h + (g + 8) * SH + c) = pack_bf16(b.x, b.y);
-    }
-}
-
 // The next layer's left operand from a layer's accumulators: GELU, rounded to BF16.
 __device__ __forceinline__ void gelu_frags(const float (*acc)[4], unsigned (*h)[4])
 {
@@ -534,23 +521,23 @@ __device__ __forceinline__ void gelu_frags(const float (*acc)[4], unsigned (*h)[
         }
 }
 
-// acc[nt][4] += H[16 x 64] (fragments) x Bt[8 NT x 64]^T (row stride SH)
-template <int NT>
-__device__ __forceinline__ void frag_gemm(const unsigned (*h)[4], const __nv_bfloat16 *Bt, float (*acc)[4], int lane)
+// acc[nt][4] += H[16 x 16 KS] (fragments) x Bt[8 NT x 16 KS]^T (row stride sb)
+template <int KS, int NT>
+__device__ __forceinline__ void frag_gemm(const unsigned (*h)[4], const __nv_bfloat16 *Bt, int sb, float (*acc)[4], int lane)
 {
     const int mi = lane >> 3, r8 = lane & 7;
 #pragma unroll
-    for (int ks = 0; ks < 4; ++ks) {
+    for (int ks = 0; ks < KS; ++ks) {
 #pragma unroll
         for (int np = 0; np < NT / 2; ++np) {
             unsigned b0, b1, b2, b3;
-            ldsm_x4(Bt + (np * 16 + (mi >> 1) * 8 + r8) * SH + ks * 16 + (mi & 1) * 8, b0, b1, b2, b3);
+            ldsm_x4(Bt + (np * 16 + (mi >> 1) * 8 + r8) * sb + ks * 16 + (mi & 1) * 8, b0, b1, b2, b3);
             mma_bf16(acc[2 * np], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b0, b1);
             mma_bf16(acc[2 * np + 1], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b2, b3);
         }
         if (NT & 1) {
             unsigned b0, b1;
-            ldsm_x2(Bt + ((NT - 1) * 8 + r8) * SH + ks * 16 + (mi & 1) * 8, b0, b1);
+            ldsm_x2(Bt + ((NT - 1) * 8 + r8) * sb + ks * 16 + (mi & 1) * 8, b0, b1);
             mma_bf16(acc[NT - 1], h[ks][0], h[ks][1], h[ks][2], h[ks][3], b0, b1);
         }
     }
@@ -572,7 +559,7 @@ struct TcGeom {
                             XA = size_t(16) * SX * 2, YS = size_t(16) * LY * 4, // a warp's input rows, y'
                             WARP = ((XA > YS ? XA : YS) + 15) / 16 * 16, TOTAL = FOLD + TC_WARPS * WARP;
 };
-constexpr size_t kFoldMaxBytes = 64 * 1024;
+constexpr size_t kFoldMaxBytes = 128 * 1024;
 
 // The BF16 weights, the folded last layer and the tables in the layout of apply_tc_kernel's
 // shared memory; one thread per element, the projections (W3 V^T)[64][4], (V b3)[4] once per CTA.
@@ -734,11 +721,11 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsign
         warp_gemm<Gm::KS1, 8>(xa, SX, w1t, SX, acc, lane);
         gelu_frags(acc, h);
         bias_init(acc, bias + 64, 8, lane);
-        frag_gemm<8>(h, w2t, acc, lane);
+        frag_gemm<4, 8>(h, w2t, SH, acc, lane);
         gelu_frags(acc, h);
         bias_init(acc, bias + 128, Gm::NT3, lane);
-        frag_gemm<Gm::NT3>(h, w3h, acc, lane);
-        frag_gemm<Gm::NT3>(h, w3l, acc, lane);
+        frag_gemm<4, Gm::NT3>(h, w3h, SH, acc, lane);
+        frag_gemm<4, Gm::NT3>(h, w3l, SH, acc, lane);
         __syncwarp(); // every lane has read its input rows
 #pragma unroll
         for (int nt = 0; nt < Gm::NT3; ++nt) { // rows g (u = 0, 1) and g + 8 (u = 2, 3)
@@ -792,18 +779,23 @@ FoldKernel fold_kernel_of(int N, int K)
 // warps takes tiles of TR_SITES columns of the feature matrix (persistent
 // over the batch); warp w owns rows 16w..16w+15 of the tile.
 //
-// per warp:  x -> z1 = x W1 + b1 -> h1 = GELU -> z2 -> h2 -> y  (mma.sync, z in
-//            registers); dY = 2 (y - t) / (count O); dz2 = (dY W3^T) GELU'(z2);
-//            dz1 = (dz2 W2^T) GELU'(z1) (mma.sync; the accumulators of the
-//            products share the fragment layout of z, so the derivative is
-//            applied in registers).  The layer inputs x, h1, h2 and the deltas
-//            dY, dz2, dz1 are rounded to BF16 as they enter a product.
+// per warp:  x -> z1 = x W1 + b1 -> h1 = GELU -> z2 -> h2 -> y (mma.sync); dY = 2 (y - t) /
+//            (count O); dz2 = (dY W3^T) GELU'(z2); dz1 = (dz2 W2^T) GELU'(z1).  The
+//            accumulators of a product have the layout of the next product's left operand,
+//            so the chain stays in registers; GELU and GELU' share their exponential and
+//            reciprocal, and GELU'(z) takes the place of z.  The layer inputs x, h1, h2 and
+//            the deltas dY, dz2, dz1 are rounded to BF16 as they enter a product.
 // per CTA:   the weight gradients gW3 = h2^T dY, gW2 = h1^T dz2, gW1 = x^T dz1
-//            are reductions over the tile's sites: their 16 x 8 blocks are
-//            spread over the warps, fragments taken transposed (ldmatrix.trans)
-//            from the row-major tile buffers, and accumulated in registers over
-//            all of the CTA's tiles; bias gradients are column sums (FP32) in
-//            shared memory.  Both go to the global gradient once per CTA.
+//            are reductions over the tile's sites: strips of 16 rows x 32 columns (40 where
+//            gW3's column tiles are odd) are spread over the warps, fragments taken
+//            transposed (ldmatrix.trans) from the row-major tile buffers, and accumulated
+//            in registers over all of the CTA's tiles.  Bias gradients are column sums
+//            (FP32): a warp's rows by a reduce-scatter over the lanes (a third of the
+//            shuffles of separate sums), the tiles in registers.  Both go to the global
+//            gradient once per CTA, two floats per reduction.
+//
+// With one CTA per SM in step between barriers, latency counts: a tile's targets are
+// loaded before its first product, the next tile's inputs before the weight gradients.
 constexpr int TR_WARPS = 8;
 constexpr int TR_SITES = 16 * TR_WARPS;
 
@@ -821,61 +813,148 @@ __device__ __forceinline__ void ldsm_x2_t(const void *p, unsigned &r0, unsigned 
                  : "r"(smem_addr(p)));
 }
 
+__device__ __forceinline__ void red_add2(float *p, float a, float b)
+{
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+
 template <int N, int K>
 struct TrGeom {
+    using Tc = TcGeom<N, K>;
     static constexpr int NPOP = (N + 1) * K, F = 10 + NPOP, O = NPOP;
     static constexpr int KS1 = (F + 15) / 16, FP = 16 * KS1, SX = FP + 8;
     static constexpr int NT3 = O / 8, OP = 16 * ((O + 15) / 16), SO = OP + 8, KS3 = OP / 16;
-    static constexpr int NB = 4 * NT3 + 32 + 8 * KS1;     // weight-gradient blocks
-    static constexpr int NBW = (NB + TR_WARPS - 1) / TR_WARPS; // per warp
+    // strips of the weight gradients: 4 x 2 of gW3 (NT3 / 2 column tiles, the second one more
+    // if odd), 4 x 2 of gW2, KS1 x 2 of gW1 (4 column tiles); a warp's blocks
+    static constexpr int NS = 16 + 2 * KS1, NSW = (NS + TR_WARPS - 1) / TR_WARPS, NTS = (NT3 + 1) / 2 > 4 ? (NT3 + 1) / 2 : 4;
+    // W1^T and W2^T as in TcGeom, then (fold_kernel, from PREP in its buffer) W2, W3^T, W3, b1 b2 b3
     static constexpr size_t W1T = 0, W2T = W1T + size_t(64) * SX * 2, W2N = W2T + size_t(64) * SH * 2,
                             W3T = W2N + size_t(64) * SH * 2, W3N = W3T + size_t(O) * SH * 2,
-                            BIAS = W3N + size_t(64) * SO * 2, GB = BIAS + size_t(128 + OP) * 4,
-                            XA = GB + size_t(128 + OP) * 4, H1 = XA + size_t(TR_SITES) * SX * 2,
+                            BIAS = W3N + size_t(64) * SO * 2, XA = (BIAS + size_t(128 + OP) * 4 + 15) / 16 * 16,
+                            H1 = XA + size_t(TR_SITES) * SX * 2,
                             H2 = H1 + size_t(TR_SITES) * SH * 2, DY = H2 + size_t(TR_SITES) * SH * 2,
                             D2 = DY + size_t(TR_SITES) * SO * 2, D1 = D2 + size_t(TR_SITES) * SH * 2,
                             TOTAL = D1 + size_t(TR_SITES) * SH * 2;
+    static constexpr size_t PREP = Tc::FOLD, PREP_END = PREP + (XA - W2N);
+    static_assert(W2N == Tc::W3H && W2T == Tc::W2, "the first two weights are shared");
+    static_assert(PREP_END <= kFoldMaxBytes, "fold buffer");
 };
 
-// rows g, g+8 of a 16 x 64 fragment set, as BF16, into a row-major tile (stride SH);
-// FP32 column sums of the 16 rows added to colsum[]
-__device__ __forceinline__ void store_rows_colsum(float (*acc)[4], __nv_bfloat16 *h, float *colsum, int lane)
+// The training kernel's copies of the weights, after apply_tc_kernel's (fold_kernel).
+template <int N, int K>
+__global__ void __launch_bounds__(256) prep_kernel(Net net, unsigned char *fold)
+{
+    using Gm = TrGeom<N, K>;
+    constexpr int O = Gm::O, SO = Gm::SO, OP = Gm::OP;
+    unsigned char *p = fold + Gm::PREP;
+    __nv_bfloat16 *w2n = reinterpret_cast<__nv_bfloat16 *>(p);
+    __nv_bfloat16 *w3t = reinterpret_cast<__nv_bfloat16 *>(p + (Gm::W3T - Gm::W2N));
+    __nv_bfloat16 *w3n = reinterpret_cast<__nv_bfloat16 *>(p + (Gm::W3N - Gm::W2N));
+    float *bias = reinterpret_cast<float *>(p + (Gm::BIAS - Gm::W2N));
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
+    for (int e = t0; e < 64 * SH; e += nt) w2n[e] = e % SH < H ? net.W2[(e / SH) * H + e % SH] : zero;
+    for (int e = t0; e < O * SH; e += nt) w3t[e] = e % SH < H ? net.W3[(e % SH) * O + e / SH] : zero;
+    for (int e = t0; e < 64 * SO; e += nt) w3n[e] = e % SO < O ? net.W3[(e / SO) * O + e % SO] : zero;
+    for (int e = t0; e < 128 + OP; e += nt)
+        bias[e] = e < 64 ? net.b1[e] : e < 128 ? net.b2[e - 64] : (e - 128 < O ? net.b3[e - 128] : 0.f);
+}
+
+// GELU of two values (as gelu2) and its derivative Phi(x) + x exp(-x^2 / 2) / sqrt(2 pi)
+__device__ __forceinline__ float2 gelu2_grad(float2 x, float2 &grad)
+{
+    constexpr float P = 0.3275911f * 0.70710678118654752f;
+    const float2 den = __ffma2_rn(make_float2(P, P), make_float2(fabsf(x.x), fabsf(x.y)), make_float2(1.f, 1.f));
+    const float2 a = __fmul2_rn(__fmul2_rn(x, x), make_float2(-0.72134752044448170f, -0.72134752044448170f));
+    float2 t, e;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(den.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(den.y));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(a.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(a.y));
+    float2 q = __ffma2_rn(make_float2(0.5f * 1.061405429f, 0.5f * 1.061405429f), t,
+                          make_float2(0.5f * -1.453152027f, 0.5f * -1.453152027f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * 1.421413741f, 0.5f * 1.421413741f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * -0.284496736f, 0.5f * -0.284496736f));
+    q = __ffma2_rn(q, t, make_float2(0.5f * 0.254829592f, 0.5f * 0.254829592f));
+    q = __fmul2_rn(__fmul2_rn(q, t), e); // 1 - Phi(|x|)
+    const float2 phi = make_float2(x.x >= 0.f ? 1.f - q.x : q.x, x.y >= 0.f ? 1.f - q.y : q.y);
+    grad = __ffma2_rn(__fmul2_rn(x, e), make_float2(0.39894228040143268f, 0.39894228040143268f), phi);
+    return __fmul2_rn(x, phi);
+}
+
+// A layer's accumulators z: GELU(z) as the next left operand h and as rows g, g + 8 of the
+// tile buffer, GELU'(z) in the place of z.
+__device__ __forceinline__ void gelu_frags_grad(float (*z)[4], unsigned (*h)[4], __nv_bfloat16 *rows, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int c = nt * 8 + t * 2;
-        *reinterpret_cast<unsigned *>(h + g * SH + c) = pack_bf16(acc[nt][0], acc[nt][1]);
-        *reinterpret_cast<unsigned *>(h + (g + 8) * SH + c) = pack_bf16(acc[nt][2], acc[nt][3]);
-        float c0 = acc[nt][0] + acc[nt][2], c1 = acc[nt][1] + acc[nt][3];
+    for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+        for (int u = 0; u < 2; ++u) {
+            float2 d;
+            const float2 v = gelu2_grad(make_float2(z[nt][2 * u], z[nt][2 * u + 1]), d);
+            z[nt][2 * u] = d.x;
+            z[nt][2 * u + 1] = d.y;
+            const unsigned b = pack_bf16(v.x, v.y);
+            h[nt >> 1][2 * (nt & 1) + u] = b;
+            *reinterpret_cast<unsigned *>(rows + (g + 8 * u) * SH + nt * 8 + 2 * t) = b;
         }
-        if (g == 0) {
-            atomicAdd(&colsum[c], c0);
-            atomicAdd(&colsum[c + 1], c1);
+}
+
+// A delta's accumulators as the next left operand and as rows of the tile buffer (stride sr)
+template <int NT>
+__device__ __forceinline__ void delta_frags(const float (*d)[4], unsigned (*h)[4], __nv_bfloat16 *rows, int sr, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const unsigned b = pack_bf16(d[nt][2 * u], d[nt][2 * u + 1]);
+            h[nt >> 1][2 * (nt & 1) + u] = b;
+            *reinterpret_cast<unsigned *>(rows + (g + 8 * u) * sr + nt * 8 + 2 * t) = b;
+        }
+}
+
+// Column sums over a warp's 16 rows, eight column tiles (those from NT on are zero): lane
+// (g, t) adds columns 8 g + 2 t, 8 g + 2 t + 1 to acc.
+template <int NT>
+__device__ __forceinline__ void column_sums(const float (*d)[4], float2 &acc, int lane)
+{
+    float c[16];
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) c[2 * nt + u] = nt < NT ? d[nt < NT ? nt : 0][u] + d[nt < NT ? nt : 0][u + 2] : 0.f;
+#pragma unroll
+    for (int n = 8, o = 16; n >= 2; n >>= 1, o >>= 1) { // keep the half that belongs to this lane's bit
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < n; ++j) {
+            const float keep = up ? c[n + j] : c[j], give = up ? c[j] : c[n + j];
+            c[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
     }
+    acc.x += c[0];
+    acc.y += c[1];
 }
 
 template <int N, int K>
 __global__ void __launch_bounds__(TR_WARPS * 32, 1)
-    train_tc_kernel(Net net, const float *__restrict__ X, const float *__restrict__ T, long long ld, long long off,
-                    int count, float inv_count, float *__restrict__ grad, float *__restrict__ loss)
+    train_tc_kernel(const unsigned char *__restrict__ fold, const float *__restrict__ X, const float *__restrict__ T,
+                    long long ld, long long off, int count, float inv_count, float *__restrict__ grad, float *__restrict__ loss)
 {
     using Gm = TrGeom<N, K>;
-    constexpr int F = Gm::F, O = Gm::O, SX = Gm::SX, SO = Gm::SO, NT3 = Gm::NT3, OP = Gm::OP, FP = Gm::FP;
-    static_assert(O % 8 == 0 && O <= 128, "output geometry");
+    constexpr int F = Gm::F, O = Gm::O, SX = Gm::SX, SO = Gm::SO, NT3 = Gm::NT3, FP = Gm::FP, NTS = Gm::NTS;
+    static_assert(O % 8 == 0 && O <= 80 && F % 2 == 0, "output geometry");
+    static_assert(TR_WARPS == 8, "a warp's first strip is of gW3, its second of gW2");
     extern __shared__ __align__(16) unsigned char sm[];
-    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W1T); // [64][SX]  W1^T
-    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W2T); // [64][SH]  W2^T
-    __nv_bfloat16 *w2n = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W2N); // [64][SH]  W2
-    __nv_bfloat16 *w3t = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W3T); // [O][SH]   W3^T
-    __nv_bfloat16 *w3n = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::W3N); // [64][SO]  W3
-    float *bias = reinterpret_cast<float *>(sm + Gm::BIAS);               // b1 | b2 | b3
-    float *gbs = reinterpret_cast<float *>(sm + Gm::GB);                  // bias gradients
+    const __nv_bfloat16 *w1t = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W1T); // [64][SX]  W1^T
+    const __nv_bfloat16 *w2t = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W2T); // [64][SH]  W2^T
+    const __nv_bfloat16 *w2n = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W2N); // [64][SH]  W2
+    const __nv_bfloat16 *w3t = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W3T); // [O][SH]   W3^T
+    const __nv_bfloat16 *w3n = reinterpret_cast<const __nv_bfloat16 *>(sm + Gm::W3N); // [64][SO]  W3
+    const float *bias = reinterpret_cast<const float *>(sm + Gm::BIAS);               // b1 | b2 | b3
     __nv_bfloat16 *xa = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::XA);   // [TR_SITES][SX]
     __nv_bfloat16 *h1b = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::H1);  // [TR_SITES][SH]
     __nv_bfloat16 *h2b = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::H2);
@@ -883,137 +962,156 @@ __global__ void __launch_bounds__(TR_WARPS * 32, 1)
     __nv_bfloat16 *d2b = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::D2);  // [TR_SITES][SH]
     __nv_bfloat16 *d1b = reinterpret_cast<__nv_bfloat16 *>(sm + Gm::D1);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    for (int e = tid; e < 64 * SX; e += blockDim.x) {
-        const int n = e / SX, k = e % SX;
-        w1t[e] = (k < F) ? net.W1[k * H + n] : zero;
-    }
-    for (int e = tid; e < 64 * SH; e += blockDim.x) {
-        const int n = e / SH, k = e % SH;
-        w2t[e] = (k < H) ? net.W2[k * H + n] : zero;
-        w2n[e] = (k < H) ? net.W2[n * H + k] : zero;
-    }
-    for (int e = tid; e < O * SH; e += blockDim.x) {
-        const int n = e / SH, k = e % SH;
-        w3t[e] = (k < H) ? net.W3[k * O + n] : zero;
-    }
-    for (int e = tid; e < 64 * SO; e += blockDim.x) {
-        const int n = e / SO, k = e % SO;
-        w3n[e] = (k < O) ? net.W3[n * O + k] : zero;
-    }
-    for (int e = tid; e < 128 + OP; e += blockDim.x) {
-        bias[e] = e < 64 ? net.b1[e] : e < 128 ? net.b2[e - 64] : (e - 128 < O ? net.b3[e - 128] : 0.f);
-        gbs[e] = 0.f;
-    }
-    for (int e = tid; e < TR_SITES * SO; e += blockDim.x) dyb[e] = zero; // columns O..SO-1 stay zero
+    const long long ntile = (count + TR_SITES - 1) / TR_SITES;
+    const int ls = lane & 15, half = lane >> 4;
+    // this lane's inputs of a tile: site ls of the warp's 16, features 4 m + 2 half, 4 m + 2 half + 1
+    float xv[FP / 2];
+    auto load_x = [&](long long tile) {
+        const long long sc = tile * TR_SITES + wid * 16 + ls;
+        const bool v = sc < count;
+        const float *p = X + 2 * half * ld + off + (v ? sc : 0);
+#pragma unroll
+        for (int m = 0; m < FP / 2; m += 2, p += 4 * ld) {
+            const bool in = v && 2 * m + 2 * half < F; // F is even
+            xv[m] = in ? p[0] : 0.f;
+            xv[m + 1] = in ? p[ld] : 0.f;
+        }
+    };
+    load_x(blockIdx.x);
+    for (int e = tid; e < int(Gm::W2N / 16); e += TR_WARPS * 32)
+        reinterpret_cast<uint4 *>(sm)[e] = __ldg(reinterpret_cast<const uint4 *>(fold) + e);
+    for (int e = tid; e < int((Gm::XA - Gm::W2N) / 16); e += TR_WARPS * 32)
+        reinterpret_cast<uint4 *>(sm + Gm::W2N)[e] = __ldg(reinterpret_cast<const uint4 *>(fold + Gm::PREP) + e);
+    for (int e = tid; e < TR_SITES * SO; e += TR_WARPS * 32) dyb[e] = __float2bfloat16_rn(0.f); // columns O.. stay zero
     __syncthreads();
 
-    float ga[Gm::NBW][4];
+    float ga[Gm::NSW][NTS][4];
 #pragma unroll
-    for (int i = 0; i < Gm::NBW; ++i)
+    for (int i = 0; i < Gm::NSW; ++i)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) ga[i][u] = 0.f;
+        for (int j = 0; j < NTS; ++j)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ga[i][j][u] = 0.f;
+    float2 gb1a = make_float2(0.f, 0.f), gb2a = gb1a, gb3a = gb1a, gb3b = gb1a;
     float lsum = 0.f;
     const int g8 = lane >> 2, t4 = lane & 3, mi = lane >> 3, r8 = lane & 7;
-    const long long ntile = (count + TR_SITES - 1) / TR_SITES;
     for (long long tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
         const long long s0 = tile * TR_SITES + wid * 16; // the warp's first column (relative to off)
         __nv_bfloat16 *xr = xa + wid * 16 * SX, *h1r = h1b + wid * 16 * SH, *h2r = h2b + wid * 16 * SH;
         __nv_bfloat16 *dyr = dyb + wid * 16 * SO, *d2r = d2b + wid * 16 * SH, *d1r = d1b + wid * 16 * SH;
-        {   // input rows (BF16), zero beyond F and beyond the batch
-            const int ls = lane & 15, half = lane >> 4;
-            const long long sc = s0 + ls;
-            const bool v = sc < count;
-            for (int f = half; f < FP; f += 2)
-                xr[ls * SX + f] = __float2bfloat16_rn(v && f < F ? X[(long long)f * ld + off + sc] : 0.f);
-        }
-        __syncwarp();
-        float z1[8][4], z2[8][4], y[NT3][4];
-        bias_init(z1, bias, 8, lane);
-        warp_gemm<Gm::KS1, 8>(xr, SX, w1t, SX, z1, lane);
-        gelu_rows(z1, h1r, lane);
-        __syncwarp();
-        bias_init(z2, bias + 64, 8, lane);
-        warp_gemm<4, 8>(h1r, SH, w2t, SH, z2, lane);
-        gelu_rows(z2, h2r, lane);
-        __syncwarp();
-        bias_init(y, bias + 128, NT3, lane);
-        warp_gemm<4, NT3>(h2r, SH, w3t, SH, y, lane);
-        // loss and dY = 2 (y - t) / (count O); rows g8 (u = 0, 1) and g8 + 8 (u = 2, 3)
+#pragma unroll
+        for (int m = 0; m < FP / 2; m += 2) // zero beyond F
+            *reinterpret_cast<unsigned *>(xr + ls * SX + 2 * m + 2 * half) = pack_bf16(xv[m], xv[m + 1]);
+        // the targets at the outputs' places: rows g8 (u = 0, 1) and g8 + 8 (u = 2, 3)
         const long long sa = s0 + g8, sb = sa + 8;
         const bool va = sa < count, vb = sb < count;
+        float y[NT3][4];
+        {
+            const float *p = T + 2 * t4 * ld + off, *pa = p + (va ? sa : 0), *pb = p + (vb ? sb : 0);
 #pragma unroll
-        for (int nt = 0; nt < NT3; ++nt) {
-            const int c = nt * 8 + 2 * t4;
-            const float d0 = va ? y[nt][0] - T[(long long)c * ld + off + sa] : 0.f;
-            const float d1 = va ? y[nt][1] - T[(long long)(c + 1) * ld + off + sa] : 0.f;
-            const float d2 = vb ? y[nt][2] - T[(long long)c * ld + off + sb] : 0.f;
-            const float d3 = vb ? y[nt][3] - T[(long long)(c + 1) * ld + off + sb] : 0.f;
-            lsum += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
-            const float q = 2.f * inv_count;
-            y[nt][0] = q * d0; y[nt][1] = q * d1; y[nt][2] = q * d2; y[nt][3] = q * d3;
-            *reinterpret_cast<unsigned *>(dyr + g8 * SO + c) = pack_bf16(y[nt][0], y[nt][1]);
-            *reinterpret_cast<unsigned *>(dyr + (g8 + 8) * SO + c) = pack_bf16(y[nt][2], y[nt][3]);
-            float c0 = y[nt][0] + y[nt][2], c1 = y[nt][1] + y[nt][3];
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) {
-                c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-                c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            }
-            if (g8 == 0) {
-                atomicAdd(&gbs[128 + c], c0);
-                atomicAdd(&gbs[128 + c + 1], c1);
+            for (int nt = 0; nt < NT3; ++nt, pa += 8 * ld, pb += 8 * ld) {
+                y[nt][0] = *pa;
+                y[nt][1] = pa[ld];
+                y[nt][2] = *pb;
+                y[nt][3] = pb[ld];
             }
         }
         __syncwarp();
+        float z1[8][4], z2[8][4];
+        unsigned h[Gm::KS3 > 4 ? Gm::KS3 : 4][4];
+        bias_init(z1, bias, 8, lane);
+        warp_gemm<Gm::KS1, 8>(xr, SX, w1t, SX, z1, lane);
+        gelu_frags_grad(z1, h, h1r, lane);
+        bias_init(z2, bias + 64, 8, lane);
+        frag_gemm<4, 8>(h, w2t, SH, z2, lane);
+        gelu_frags_grad(z2, h, h2r, lane);
+#pragma unroll
+        for (int nt = 0; nt < NT3; ++nt) { // y - t from the start
+            const float2 b = *reinterpret_cast<const float2 *>(bias + 128 + nt * 8 + 2 * t4);
+            y[nt][0] = b.x - y[nt][0];
+            y[nt][1] = b.y - y[nt][1];
+            y[nt][2] = b.x - y[nt][2];
+            y[nt][3] = b.y - y[nt][3];
+        }
+        frag_gemm<4, NT3>(h, w3t, SH, y, lane);
+        // loss and dY = 2 (y - t) / (count O)
+        const float q = 2.f * inv_count;
+#pragma unroll
+        for (int nt = 0; nt < NT3; ++nt)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float d = (u < 2 ? va : vb) ? y[nt][u] : 0.f;
+                lsum += d * d;
+                y[nt][u] = q * d;
+            }
+        column_sums<(NT3 < 8 ? NT3 : 8)>(y, gb3a, lane);
+        if constexpr (NT3 > 8) { // the ninth column tile, summed over its rows at the end
+            gb3b.x += y[8][0] + y[8][2];
+            gb3b.y += y[8][1] + y[8][3];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[Gm::KS3 - 1][u] = 0u; // an odd column tile's other half
+        delta_frags<NT3>(y, h, dyr, SO, lane);
         // dz2 = (dY W3^T) GELU'(z2)
         float da[8][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
             for (int u = 0; u < 4; ++u) da[nt][u] = 0.f;
-        warp_gemm<Gm::KS3, 8>(dyr, SO, w3n, SO, da, lane);
+        frag_gemm<Gm::KS3, 8>(h, w3n, SO, da, lane);
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) da[nt][u] *= gelu_grad(z2[nt][u]);
-        store_rows_colsum(da, d2r, gbs + 64, lane);
-        __syncwarp();
+            for (int u = 0; u < 4; ++u) da[nt][u] *= z2[nt][u];
+        column_sums<8>(da, gb2a, lane);
+        delta_frags<8>(da, h, d2r, SH, lane);
         // dz1 = (dz2 W2^T) GELU'(z1)
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
             for (int u = 0; u < 4; ++u) da[nt][u] = 0.f;
-        warp_gemm<4, 8>(d2r, SH, w2n, SH, da, lane);
+        frag_gemm<4, 8>(h, w2n, SH, da, lane);
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) da[nt][u] *= gelu_grad(z1[nt][u]);
-        store_rows_colsum(da, d1r, gbs, lane);
+            for (int u = 0; u < 4; ++u) da[nt][u] *= z1[nt][u];
+        column_sums<8>(da, gb1a, lane);
+        delta_frags<8>(da, h, d1r, SH, lane);
         __syncthreads();
-        // weight-gradient blocks over the tile's TR_SITES sites
+        if (tile + gridDim.x < ntile) load_x(tile + gridDim.x);
+        // weight-gradient strips over the tile's TR_SITES sites
 #pragma unroll
-        for (int i = 0; i < Gm::NBW; ++i) {
+        for (int i = 0; i < Gm::NSW; ++i) {
             const int b = wid + TR_WARPS * i;
-            if (b < Gm::NB) {
+            if (b < Gm::NS) {
                 const __nv_bfloat16 *As, *Bs;
-                int sa_, sb_, m0, n0;
-                if (b < 4 * NT3) {
-                    As = h2b; sa_ = SH; Bs = dyb; sb_ = SO; m0 = (b / NT3) * 16; n0 = (b % NT3) * 8;
-                } else if (b < 4 * NT3 + 32) {
-                    const int bb = b - 4 * NT3;
-                    As = h1b; sa_ = SH; Bs = d2b; sb_ = SH; m0 = (bb / 8) * 16; n0 = (bb % 8) * 8;
+                int sa_, sb_, m0 = (b >> 1) * 16, n0 = (b & 1) * 32, nts = 4;
+                if (i == 0) {
+                    As = h2b; sa_ = SH; Bs = dyb; sb_ = SO; n0 = (b & 1) * (NT3 / 2) * 8; nts = (b & 1) ? NT3 - NT3 / 2 : NT3 / 2;
+                } else if (i == 1) {
+                    As = h1b; sa_ = SH; Bs = d2b; sb_ = SH; m0 -= 64;
                 } else {
-                    const int bb = b - 4 * NT3 - 32;
-                    As = xa; sa_ = SX; Bs = d1b; sb_ = SH; m0 = (bb / 8) * 16; n0 = (bb % 8) * 8;
+                    As = xa; sa_ = SX; Bs = d1b; sb_ = SH; m0 -= 128;
                 }
+                const __nv_bfloat16 *ap = As + ((mi >> 1) * 8 + r8) * sa_ + m0 + (mi & 1) * 8;
+                const __nv_bfloat16 *bp = Bs + ((mi & 1) * 8 + r8) * sb_ + n0 + (mi >> 1) * 8;
 #pragma unroll
                 for (int ks = 0; ks < TR_SITES / 16; ++ks) {
-                    const int k0 = ks * 16;
-                    unsigned a0, a1, a2, a3, b0, b1;
-                    ldsm_x4_t(As + (k0 + (mi >> 1) * 8 + r8) * sa_ + m0 + (mi & 1) * 8, a0, a1, a2, a3);
-                    ldsm_x2_t(Bs + (k0 + (mi & 1) * 8 + r8) * sb_ + n0, b0, b1);
-                    mma_bf16(ga[i], a0, a1, a2, a3, b0, b1);
+                    unsigned a0, a1, a2, a3;
+                    ldsm_x4_t(ap + ks * 16 * sa_, a0, a1, a2, a3);
+#pragma unroll
+                    for (int j = 0; j < NTS; j += 2) {
+                        if (j + 1 < nts) {
+                            unsigned b0, b1, b2, b3; // column tiles j and j + 1
+                            ldsm_x4_t(bp + ks * 16 * sb_ + j * 8, b0, b1, b2, b3);
+                            mma_bf16(ga[i][j], a0, a1, a2, a3, b0, b1);
+                            if (j + 1 < NTS) mma_bf16(ga[i][j + 1 < NTS ? j + 1 : j], a0, a1, a2, a3, b2, b3);
+                        } else if (j < nts) {
+                            unsigned b0, b1;
+                            ldsm_x2_t(bp + ks * 16 * sb_ + j * 8, b0, b1);
+                            mma_bf16(ga[i][j], a0, a1, a2, a3, b0, b1);
+                        }
+                    }
                 }
             }
         }
@@ -1022,39 +1120,69 @@ __global__ void __launch_bounds__(TR_WARPS * 32, 1)
     // the CTA's contributions to the global gradient (layout W1 [F][H] | b1 | W2 [H][H] | b2 | W3 [H][O] | b3)
     float *gW1 = grad, *gb1 = gW1 + F * H, *gW2 = gb1 + H, *gb2 = gW2 + H * H, *gW3 = gb2 + H, *gb3 = gW3 + H * O;
 #pragma unroll
-    for (int i = 0; i < Gm::NBW; ++i) {
+    for (int i = 0; i < Gm::NSW; ++i) {
         const int b = wid + TR_WARPS * i;
-        if (b >= Gm::NB) continue;
-        int m0, n0, which;
-        if (b < 4 * NT3) { which = 3; m0 = (b / NT3) * 16; n0 = (b % NT3) * 8; }
-        else if (b < 4 * NT3 + 32) { which = 2; m0 = ((b - 4 * NT3) / 8) * 16; n0 = ((b - 4 * NT3) % 8) * 8; }
-        else { which = 1; m0 = ((b - 4 * NT3 - 32) / 8) * 16; n0 = ((b - 4 * NT3 - 32) % 8) * 8; }
+        if (b >= Gm::NS) continue;
+        int m0 = (b >> 1) * 16, n0 = (b & 1) * 32, nts = 4, width = H, rows = H;
+        float *gw = gW2;
+        if (i == 0) {
+            gw = gW3; width = O; n0 = (b & 1) * (NT3 / 2) * 8; nts = (b & 1) ? NT3 - NT3 / 2 : NT3 / 2;
+        } else if (i == 1) {
+            m0 -= 64;
+        } else {
+            gw = gW1; m0 -= 128; rows = F;
+        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int m = m0 + g8 + (u < 2 ? 0 : 8), n = n0 + 2 * t4 + (u & 1);
-            if (which == 3) atomicAdd(&gW3[m * O + n], ga[i][u]);
-            else if (which == 2) atomicAdd(&gW2[m * H + n], ga[i][u]);
-            else if (m < F) atomicAdd(&gW1[m * H + n], ga[i][u]);
+        for (int j = 0; j < NTS; ++j) {
+            if (j >= nts) continue;
+            float *p = gw + (m0 + g8) * width + n0 + j * 8 + 2 * t4;
+            if (m0 + g8 < rows) red_add2(p, ga[i][j][0], ga[i][j][1]);
+            if (m0 + g8 + 8 < rows) red_add2(p + 8 * width, ga[i][j][2], ga[i][j][3]);
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     if (lane == 0) atomicAdd(loss, lsum);
+    // bias gradients: the warps' sums through shared memory (the loop ended with a barrier)
+    float *gbs = reinterpret_cast<float *>(h1b); // [TR_WARPS][128 + 80]
+    constexpr int GB = 128 + 80;
+    float *own = gbs + wid * GB;
+    const int col = 8 * g8 + 2 * t4;
+    *reinterpret_cast<float2 *>(own + col) = gb1a;
+    *reinterpret_cast<float2 *>(own + 64 + col) = gb2a;
+    *reinterpret_cast<float2 *>(own + 128 + col) = gb3a;
+    if constexpr (NT3 > 8) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            gb3b.x += __shfl_xor_sync(0xffffffffu, gb3b.x, o);
+            gb3b.y += __shfl_xor_sync(0xffffffffu, gb3b.y, o);
+        }
+        if (g8 == 0) *reinterpret_cast<float2 *>(own + 192 + 2 * t4) = gb3b;
+    }
     __syncthreads();
-    for (int e = tid; e < 128 + O; e += blockDim.x) {
-        if (e < 64) atomicAdd(&gb1[e], gbs[e]);
-        else if (e < 128) atomicAdd(&gb2[e - 64], gbs[e]);
-        else atomicAdd(&gb3[e - 128], gbs[e]);
+    for (int e = tid; e < 128 + O; e += TR_WARPS * 32) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < TR_WARPS; ++w) v += gbs[w * GB + e];
+        atomicAdd(e < 64 ? gb1 + e : e < 128 ? gb2 + (e - 64) : gb3 + (e - 128), v);
     }
 }
 
-using TrKernel = void (*)(Net, const float *, const float *, long long, long long, int, float, float *, float *);
+using TrKernel = void (*)(const unsigned char *, const float *, const float *, long long, long long, int, float, float *, float *);
+using PrepKernel = void (*)(Net, unsigned char *);
 
 TrKernel tr_kernel(int N, int K, size_t *smem)
 {
     if (N == 2 && K == 24) { *smem = TrGeom<2, 24>::TOTAL; return train_tc_kernel<2, 24>; }
     if (N == 2 && K == 16) { *smem = TrGeom<2, 16>::TOTAL; return train_tc_kernel<2, 16>; }
     if (N == 3 && K == 16) { *smem = TrGeom<3, 16>::TOTAL; return train_tc_kernel<3, 16>; }
+    return nullptr;
+}
+PrepKernel prep_kernel_of(int N, int K)
+{
+    if (N == 2 && K == 24) return prep_kernel<2, 24>;
+    if (N == 2 && K == 16) return prep_kernel<2, 16>;
+    if (N == 3 && K == 16) return prep_kernel<3, 16>;
     return nullptr;
 }
 
@@ -1070,7 +1198,8 @@ struct rlbm_closure {
     __nv_bfloat16 *d_w = nullptr;   // W1 | W2 | W3 in BF16
     int *d_wmap = nullptr;          // BF16 weight -> master index
     float *d_tab = nullptr;         // p0 | c | s | w | Ainv
-    float *d_loss = nullptr;
+    float *d_loss = nullptr;        // after the gradient: one clear and one copy serve both
+    float *h_stage = nullptr;       // pinned: gradient and loss on their way to the caller
     unsigned char *d_fold = nullptr; // weights and tables as apply_tc_kernel keeps them in shared memory
     int adam_t = 0;
     bool simt_apply = false;
@@ -1155,6 +1284,7 @@ rlbm_status refresh_bf16(rlbm_closure *c)
     CL_CUDA(c, cudaGetLastError());
     if (FoldKernel k = fold_kernel_of(c->N, c->K)) { // in stream order, also under capture
         k<<<16, 256, 0, c->stream>>>(net_of(c), tab_of(c), c->d_fold);
+        prep_kernel_of(c->N, c->K)<<<16, 256, 0, c->stream>>>(net_of(c), c->d_fold);
         CL_CUDA(c, cudaGetLastError());
     }
     return RLBM_OK;
@@ -1254,12 +1384,13 @@ rlbm_status rlbm_closure_create(rlbm_closure_t **out, int order_N, int angles_K,
         for (int i = 0; i < H * H; ++i) wmap[k++] = int(c->off_W2) + i;
         for (int i = 0; i < H * c->O; ++i) wmap[k++] = int(c->off_W3) + i;
     }
-    if (cudaMalloc(&c->d_p, c->nparam * 4) != cudaSuccess || cudaMalloc(&c->d_g, c->nparam * 4) != cudaSuccess ||
+    if (cudaMalloc(&c->d_p, c->nparam * 4) != cudaSuccess || cudaMalloc(&c->d_g, (c->nparam + 1) * 4) != cudaSuccess ||
         cudaMalloc(&c->d_m, c->nparam * 4) != cudaSuccess || cudaMalloc(&c->d_v, c->nparam * 4) != cudaSuccess ||
         cudaMalloc(&c->d_w, size_t(nw) * 2) != cudaSuccess || cudaMalloc(&c->d_wmap, size_t(nw) * 4) != cudaSuccess ||
-        cudaMalloc(&c->d_tab, tab.size() * 4) != cudaSuccess || cudaMalloc(&c->d_loss, 4) != cudaSuccess ||
-        cudaMalloc(&c->d_fold, kFoldMaxBytes) != cudaSuccess)
+        cudaMalloc(&c->d_tab, tab.size() * 4) != cudaSuccess || cudaMalloc(&c->d_fold, kFoldMaxBytes) != cudaSuccess ||
+        cudaMallocHost(&c->h_stage, (c->nparam + 1) * 4) != cudaSuccess)
         return bail(cfail(c, RLBM_ERR_OOM, "device allocation failed"));
+    c->d_loss = c->d_g + c->nparam;
     if (cudaMemcpyAsync(c->d_p, p.data(), c->nparam * 4, cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->d_m, 0, c->nparam * 4, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->d_v, 0, c->nparam * 4, c->stream) != cudaSuccess ||
@@ -1284,7 +1415,8 @@ void rlbm_closure_destroy(rlbm_closure_t *c)
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     cudaFree(c->d_p); cudaFree(c->d_g); cudaFree(c->d_m); cudaFree(c->d_v);
-    cudaFree(c->d_w); cudaFree(c->d_wmap); cudaFree(c->d_tab); cudaFree(c->d_loss); cudaFree(c->d_fold);
+    cudaFree(c->d_w); cudaFree(c->d_wmap); cudaFree(c->d_tab); cudaFree(c->d_fold);
+    if (c->h_stage) cudaFreeHost(c->h_stage);
     delete c;
 }
 
@@ -1384,12 +1516,23 @@ rlbm_status rlbm_closure_forward(rlbm_closure_t *c, const float *d_x, long long 
     return RLBM_OK;
 }
 
-// gradient of the mean-squared error over columns [off, off + count) into d_g; loss to host
-static rlbm_status closure_grad(rlbm_closure_t *c, const float *d_x, const float *d_t, long long ld, long long off,
-                                int count, float *d_z1, float *d_z2, float *d_dy, float *loss)
+// the gradient and the loss to the host, as far as they are wanted: one copy, one wait
+static rlbm_status closure_fetch(rlbm_closure_t *c, int count, float *host_grad, float *loss)
 {
-    CL_CUDA(c, cudaMemsetAsync(c->d_g, 0, c->nparam * 4, c->stream));
-    CL_CUDA(c, cudaMemsetAsync(c->d_loss, 0, 4, c->stream));
+    if (!host_grad && !loss) return RLBM_OK;
+    const size_t first = host_grad ? 0 : c->nparam;
+    CL_CUDA(c, cudaMemcpyAsync(c->h_stage + first, c->d_g + first, (c->nparam + 1 - first) * 4, cudaMemcpyDeviceToHost, c->stream));
+    CL_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (host_grad) std::memcpy(host_grad, c->h_stage, c->nparam * 4);
+    if (loss) *loss = c->h_stage[c->nparam] / (float(count) * float(c->O));
+    return RLBM_OK;
+}
+
+// gradient of the mean-squared error over columns [off, off + count) into d_g (and host_grad); loss to host
+static rlbm_status closure_grad(rlbm_closure_t *c, const float *d_x, const float *d_t, long long ld, long long off,
+                                int count, float *d_z1, float *d_z2, float *d_dy, float *host_grad, float *loss)
+{
+    CL_CUDA(c, cudaMemsetAsync(c->d_g, 0, (c->nparam + 1) * 4, c->stream));
     size_t trsmem = 0;
     TrKernel tk = c->simt_train ? nullptr : tr_kernel(c->N, c->K, &trsmem);
     if (tk) {
@@ -1399,16 +1542,10 @@ static rlbm_status closure_grad(rlbm_closure_t *c, const float *d_x, const float
         CL_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const long long tiles = (count + TR_SITES - 1) / TR_SITES;
         const int grid = int(std::min<long long>(sms, tiles));
-        tk<<<grid, TR_WARPS * 32, trsmem, c->stream>>>(net_of(c), d_x, d_t, ld, off, count,
+        tk<<<grid, TR_WARPS * 32, trsmem, c->stream>>>(c->d_fold, d_x, d_t, ld, off, count,
                                                       1.0f / (float(count) * float(c->O)), c->d_g, c->d_loss);
         CL_CUDA(c, cudaGetLastError());
-        if (loss) {
-            float l = 0.f;
-            CL_CUDA(c, cudaMemcpyAsync(&l, c->d_loss, 4, cudaMemcpyDeviceToHost, c->stream));
-            CL_CUDA(c, cudaStreamSynchronize(c->stream));
-            *loss = l / (float(count) * float(c->O));
-        }
-        return RLBM_OK;
+        return closure_fetch(c, count, host_grad, loss);
     }
     const int grid = std::min(2048, (count + 127) / 128);
     const float inv = 1.0f / (float(count) * float(c->O));
@@ -1420,27 +1557,15 @@ static rlbm_status closure_grad(rlbm_closure_t *c, const float *d_x, const float
     mlp_backward_kernel<<<std::min(tiles, 1024), 128, bwd_smem(c), c->stream>>>(net_of(c), d_x + off, ld, 0, count,
                                                                             d_z1, d_z2, d_dy, c->d_g);
     CL_CUDA(c, cudaGetLastError());
-    if (loss) {
-        float l = 0.f;
-        CL_CUDA(c, cudaMemcpyAsync(&l, c->d_loss, 4, cudaMemcpyDeviceToHost, c->stream));
-        CL_CUDA(c, cudaStreamSynchronize(c->stream));
-        *loss = l / (float(count) * float(c->O));
-    }
-    return RLBM_OK;
+    return closure_fetch(c, count, host_grad, loss);
 }
 
 rlbm_status rlbm_closure_gradient(rlbm_closure_t *c, const float *d_x, const float *d_t, long long ld, long long off,
                                   int count, float *d_work, float *host_grad, float *loss)
 {
     if (!c || !d_x || !d_t || !d_work || count < 1) return cfail(c, RLBM_ERR_ARG, "bad arguments");
-    rlbm_status st = closure_grad(c, d_x, d_t, ld, off, count, d_work, d_work + size_t(H) * ld,
-                                  d_work + size_t(2 * H) * ld, loss);
-    if (st) return st;
-    if (host_grad) {
-        CL_CUDA(c, cudaMemcpyAsync(host_grad, c->d_g, c->nparam * 4, cudaMemcpyDeviceToHost, c->stream));
-        CL_CUDA(c, cudaStreamSynchronize(c->stream));
-    }
-    return RLBM_OK;
+    return closure_grad(c, d_x, d_t, ld, off, count, d_work, d_work + size_t(H) * ld, d_work + size_t(2 * H) * ld,
+                        host_grad, loss);
 }
 
 size_t rlbm_closure_work_floats(const rlbm_closure_t *c, long long ld)
@@ -1453,7 +1578,7 @@ rlbm_status rlbm_closure_train_step(rlbm_closure_t *c, const float *d_x, const f
 {
     if (!c || !d_x || !d_t || !d_work || count < 1 || !(lr > 0.f)) return cfail(c, RLBM_ERR_ARG, "bad arguments");
     rlbm_status st = closure_grad(c, d_x, d_t, ld, off, count, d_work, d_work + size_t(H) * ld,
-                                  d_work + size_t(2 * H) * ld, loss);
+                                  d_work + size_t(2 * H) * ld, nullptr, loss);
     if (st) return st;
     ++c->adam_t;
     const float b1 = 0.9f, b2 = 0.999f;

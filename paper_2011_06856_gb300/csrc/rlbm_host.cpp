@@ -712,7 +712,7 @@ bool split_wanted(const rlbm_t *h)
 
 // Its ring and counters for the handle's present tiling (the stream is idle: creation and
 // retile).  A tile's two passes lie as many tiles apart as run at a time; the ring is three
-// times that.  Without memory the handle runs the per-tile kernel.
+// times that, or all tiles.  Without memory the handle runs the per-tile kernel.
 void setup_split(rlbm_t *h)
 {
     if (h->d_split) cudaFree(h->d_split);
@@ -729,7 +729,8 @@ void setup_split(rlbm_t *h)
     // while the tiles do not fill the GPU, of at least two quads per warp
     int cs = 1;
     while (2 * cs * (h->N + 1) <= 16 && tiles * (h->N + 1) * cs < resident && h->K / 4 >= 2 * cs * 2 * rlbmk::kSplitWarps) cs *= 2;
-    const int parts = cs * (h->N + 1), lag = (resident + parts - 1) / parts, ring = 3 * lag;
+    const int parts = cs * (h->N + 1), lag = (resident + parts - 1) / parts;
+    const int ring = int(std::min<long long>(3ll * lag, tiles));
     const size_t sync = (size_t(rlbmk::kSplitSyncWords + tiles) * 4 + 255) / 256 * 256;
     const size_t bytes = sync + size_t(ring) * rlbmk::split_tile_floats(h->N, cs) * 4;
     if (2ll * parts * tiles > 0x7fffffffll || cudaMalloc(&h->d_split, bytes) != cudaSuccess ||

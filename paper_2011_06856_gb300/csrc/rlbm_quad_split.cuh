@@ -67,15 +67,17 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
     constexpr bool DD = sizeof(St) == 4;
     using Rows = QuadRows<N, DD>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ unsigned s_ticket, s_last;
+    __shared__ unsigned s_ticket, s_abort, s_last;
     const int lane = threadIdx.x, q = warp_uniform(threadIdx.y), K4 = a.K >> 2, CS = a.split_cs, PARTS = CS * (N + 1);
     const bool first = q == 0 && lane == 0;
     float *red = reinterpret_cast<float *>(smem_raw); // [5][max(NW, PARTS)][64]
     float *sres = red + 5 * max(NW, PARTS) * kPairSites;
 
-    if (first) s_ticket = atomicAdd(a.split_sync, 1u);
+    if (first) {
+        s_ticket = atomicAdd(a.split_sync, 1u);
+        s_abort = __ldcg(a.split_sync + 3); // one read for the CTA: it may change at any time
+    }
     const unsigned seed = __ldcg(a.ctr), base = __ldcg(a.split_sync + 2) * unsigned(2 * PARTS + 1);
-    const bool aborted = __ldcg(a.split_sync + 3) != 0u;
     __syncthreads();
     // ticket -> pass, tile, part: A alone for the first lag tiles, B alone for the last
     const int lag = a.split_lag, k = warp_uniform(s_ticket), head = lag * PARTS, mid = (ntiles - lag) * 2 * PARTS;
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
     float *coef = slot + 5 * PARTS * kPairSites, *oslot = coef + (N + 1) * NC * kPairSites;
     unsigned *word = a.split_sync + kSplitSyncWords + tile;
 
-    if (aborted) {
+    if (s_abort) {
         // a wait ran out: the step is void and reported
     } else if (!passB) {
         QuadSums sums = quad_sums_zero();

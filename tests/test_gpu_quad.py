@@ -157,3 +157,24 @@ def test_many_angles_report_an_unphysical_cell():
         sim.step(1)
         with pytest.raises(R.Unphysical):
             sim.sync()
+
+
+def test_many_angles_expired_wait_is_reported_and_recovered_from():
+    """With a wait limit far below a tile's first pass the second pass gives up: the step is
+    reported, and the same handle steps correctly afterwards (its counters start over)."""
+    nx, ny, N, K = 96, 4, 3, 288
+    fl = W.random_fields(nx, ny, seed=9)
+    q = O.Quadrature(N, K)
+    ref, flagged = q.run(q.init(fl.n, fl.T, fl.bx, fl.by), 2.5, 3, OUT, PER)
+    assert flagged == 0
+    with R.Simulation(nx, ny, N, K, 2.5, "fp32", OUT, PER) as sim:
+        sim.init_fields(fl)
+        sim.set_wait_limit(1000)
+        sim.step(1)
+        with pytest.raises(R.DeviceTimeout):
+            sim.sync()
+        sim.set_wait_limit(4_000_000_000)
+        sim.init_fields(fl)
+        sim.step(3)
+        sim.sync()
+        assert relerr(sim.get_populations().astype(np.float64), ref) < FP32_TOL

@@ -392,7 +392,9 @@ __global__ void __launch_bounds__(128) apply_kernel(Net net, CoarseTab q, float 
 // sixteen warps of an SM run through loads, arithmetic, products and stores at different
 // times.  (Tiles of 192 sites through shared memory, copied a tile ahead and processed in
 // step by twelve warps between CTA barriers, took 300 us on 1024^2 sites, K = 24, N = 2, at
-// 0.4 instructions a cycle and scheduler; the populations' one read and one write take 89.)
+// 0.4 instructions a cycle and scheduler; this form 215, bound by the shared-memory reads of
+// the weights and by issue.  The populations' one read and one write take 89.  Two groups of
+// 16 sites per warp sharing the weight fragments, the populations read again: 263.)
 //
 // * Conservation folded into the last layer.  With d = n0 W y (W = diag w) the
 //   projection d - W C^T A^-1 C d equals n0 W Q y, Q = I - C^T A^-1 C W, a
@@ -650,8 +652,8 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsign
     const int g = lane >> 2, t = lane & 3;
     const int ls = lane & 15, half = lane >> 4;
     const long long ngroup = (S + 15) / 16, nwarp = (long long)gridDim.x * TC_WARPS;
-    // groups next to each other run at the same time: their rows share DRAM pages
-    for (long long group = (long long)blockIdx.x * TC_WARPS + wid; group < ngroup; group += nwarp) {
+    // a short grid's groups spread over all SMs
+    for (long long group = (long long)wid * gridDim.x + blockIdx.x; group < ngroup; group += nwarp) {
         const long long site = group * 16 + ls;
         const bool valid = site < S;
         // ---- this lane takes angles [half K/2, (half+1) K/2) of every shell of its site
@@ -737,6 +739,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsign
         // ---- update: f_i += n0 w_i y'_i
         if (valid) {
             float *p = fs;
+            asm volatile("" : "+l"(p)); // else the addresses of the loads are kept, two registers each
 #pragma unroll
             for (int r = 0; r <= N; ++r) {
 #pragma unroll
@@ -1600,8 +1603,7 @@ rlbm_status rlbm_closure_apply_buffer(rlbm_closure_t *c, float *d_f, long long s
         int dev = 0, sms = 0;
         CL_CUDA(c, cudaGetDevice(&dev));
         CL_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const long long tiles = (sites + 16 * TC_WARPS - 1) / (16 * TC_WARPS);
-        const int grid = int(std::min<long long>(sms, tiles));
+        const int grid = int(std::min<long long>(sms, (sites + 15) / 16));
         k<<<grid, TC_WARPS * 32, smem, c->stream>>>(c->d_fold, d_f, sites, float(kn));
         CL_CUDA(c, cudaGetLastError());
         return RLBM_OK;

@@ -237,7 +237,10 @@ long long rlbm_kernel_launches(const rlbm_t *h);
  * chunks of 4 or 8 populations that share sgn(v_y); row pitch a multiple of
  * 16 bytes, nx >= 64 + 32 bytes of halo, one population group; bounded
  * mbarrier wait; 16-bit stores round stochastically with cvt.rs),
- * 0 = per-tile kernel. */
+ * 0 = per-tile kernel; where N <= 3, the collision is finite and K is a
+ * multiple of 4, kind 0 also stands for the quadrant kernels for any nx (K a
+ * multiple of P in the same list) and, like kind 2, for the two-pass kernel of
+ * many angles (bounded waits on its own counters). */
 int rlbm_step_kernel_variant(const rlbm_t *h);
 
 /* Select the tiling and step kernel directly (no counterpart in the paper:
@@ -261,8 +264,9 @@ int rlbm_tile_populations(const rlbm_t *h);
  * per shell own ceil(K / (warps P)) groups each; the streamed values of all
  * but the last group are parked in the output buffer between the two passes
  * (FP32 and FP64 storage; rlbm_create refuses such K in 16-bit storage).
- * The per-tile kernel and, in FP32 storage with K a multiple of P, the
- * two-sites-per-lane kernel (without staging) apply.  -1 for a NULL handle. */
+ * FP32 storage with N <= 3 and K a multiple of 4 runs such K in the two-pass
+ * kernel instead (kind 0, and kind 2 for K a multiple of P), whatever the
+ * tiling.  -1 for a NULL handle. */
 int rlbm_population_groups(const rlbm_t *h);
 
 /* Autotuner: time every compiled tiling of the step kernel (P populations per

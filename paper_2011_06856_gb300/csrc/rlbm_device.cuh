@@ -36,6 +36,7 @@
 #include <stdint.h>
 
 #include "rlbm_args.h"
+#include "rlbm_bits.cuh"
 #include "rlbm_df64.cuh"
 #include "rlbm_stat.cuh"
 
@@ -105,15 +106,6 @@ __device__ __forceinline__ double r_div(double a, double b) { return a / b; }
 // and only random-walks.  Random bits: one hash per thread and tile (of the
 // site, the warp and the launch counter), then a 32-bit LCG step per store;
 // the top bits are added below the kept mantissa and the value truncated.
-__device__ __forceinline__ unsigned mix32(unsigned x)
-{
-    x ^= x >> 16;
-    x *= 0x7feb352du;
-    x ^= x >> 15;
-    x *= 0x846ca68bu;
-    x ^= x >> 16;
-    return x;
-}
 __device__ __forceinline__ unsigned lcg_next(unsigned &s)
 {
     s = s * 1664525u + 1013904223u;

@@ -167,13 +167,14 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
     // pass 2: this warp's shell coefficients, f^eq, relaxation (Eq. discrete-rbe), stores
     float2 cf[NC], o[3];
     quad_shell<N, DD>(a, r, r, q, Gs, sres, red, lane, cf, o);
-    QuadBits rng = quad_seed(unsigned(y * a.nx + xl), unsigned(g), seed);
+    QuadBits rng = quad_seed(unsigned(y) * unsigned(a.nx) + unsigned(xl), unsigned(g), seed);
     const long long Sb = S * (long long)sizeof(St), KS = K4 * Sb;
     char *ob = reinterpret_cast<char *>(a.fout) + i0 * Sb + ((long long)y * a.nx + (act ? xl : 0)) * int(sizeof(St));
 #pragma unroll
     for (int k = 0; k < QW; ++k) {
         float2 feq[4], om[4];
         quad_equilibrium<N>(cf, o, tb + 3 * k, feq, om);
+        if (k > 0 && 4 * k % QuadBits::kWords == 0) rng.refresh();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             char *p = ob + (k * Sb + u * KS);

@@ -456,31 +456,6 @@ __device__ __forceinline__ float2 lerp_x(float2 C, float e, float2 ax)
     return pfma(ax, d, C);
 }
 
-// Random bits of the stochastic rounding: the k-th word of a thread is the exclusive or of
-// two hashed words rotated by 5 k and 3 k bits.  Any two words are independent bit by bit
-// (no pair of bits meets twice within 32 words), which is what the moments of the rounding
-// errors need, and a word costs three integer operations on the pipe that the arithmetic
-// leaves idle; an LCG draw (IMAD) takes two cycles of the FMA pipe, a 64-bit product four.
-struct QuadBits {
-    unsigned a, b;
-    __device__ __forceinline__ unsigned next()
-    {
-        a = __funnelshift_l(a, a, 5);
-        b = __funnelshift_l(b, b, 3);
-        return a ^ b;
-    }
-};
-// Seeded by the thread's first site, the warp and the launch counter.  The site is hashed
-// before the counter enters: the exclusive or of the counter's hash with the bare site index
-// only permutes the seeds of a launch among the sites, so that every launch rounds with
-// almost the same set of words, and the mean error of that set becomes a drift of n (5e-4
-// over 2000 steps of a 256^2 grid in FP16).
-__device__ __forceinline__ QuadBits quad_seed(unsigned site, unsigned g, unsigned launch)
-{
-    const unsigned h = mix32(mix32(site * 256u + g) ^ mix32(launch * 0x9E3779B9u + 1u));
-    return {h, mix32(h + 0x9E3779B9u)};
-}
-
 // The relaxation f* + om (f^eq - f*) of two FP32 sites, rounded stochastically.  r, the
 // result rounded to nearest, gives the binade; t = om d + noise, the noise uniform in
 // +- ulp(r) / 2; f* + t is rounded once.  The rounding of t (2^-24 |om d|) is below that
@@ -757,7 +732,7 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
 
     float2 cf[NC], o[3];
     quad_shell<N, DD>(a, r, r, q, Gs, sres, red, lane, cf, o);
-    QuadBits rng = quad_seed(unsigned(t.y * a.nx + t.x), unsigned(g), seed);
+    QuadBits rng = quad_seed(unsigned(t.y) * unsigned(a.nx) + unsigned(t.x), unsigned(g), seed);
     const QuadOut<St, MAP> out(a, t, reinterpret_cast<char *>(a.fout) + i0 * Sb);
 #pragma unroll
     for (int k = 0; k < QW; ++k) {
@@ -765,6 +740,7 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
                               N == 3 ? __ldg(tb + 3 * k + 2) : make_float4(0.f, 0.f, 0.f, 0.f)};
         float2 feq[4], om[4];
         quad_equilibrium<N>(cf, o, tq, feq, om);
+        if (k > 0 && 4 * k % QuadBits::kWords == 0) rng.refresh();
         out.store(k * Sb, KS, fs + 4 * k, feq, om, rng);
     }
     __syncthreads();

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
             }
         }
     } else {
-        QuadBits rng = quad_seed(unsigned(t.y * a.nx + t.x), unsigned(part * NW + q), seed);
+        QuadBits rng = quad_seed(unsigned(t.y) * unsigned(a.nx) + unsigned(t.x), unsigned(part * NW + q), seed);
         const QuadOut<St, MAP> out(a, t, reinterpret_cast<char *>(a.fout) + pop0);
         auto passB_run = [&](auto edge_tag) {
             using Pull = QuadPull<St, MAP, TWO_D, decltype(edge_tag)::value>;
@@ -210,6 +210,9 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
                 load(j + NW); // its latency passes behind the equilibrium and the stores
                 quad_equilibrium<N>(cf, o, tq, feq, om);
                 out.store(j * Sb, KS, f, feq, om, rng);
+                constexpr int TURN = (QuadBits::kWords / 4 - 1) * NW; // the warp's fourth quad since the last one
+                static_assert((NW & (NW - 1)) == 0, "quads counted by the bits of j - j0");
+                if (((j - j0) & TURN) == TURN) rng.refresh();
             }
         };
         if (t.interior(a)) passB_run(QuadTag<false>{});

@@ -361,8 +361,9 @@ RLBM_DECLARE_PAIR_TMA(bf16)
 
 // Free streaming of thin grids (rlbm_free.cu): nsteps <= kFreeSteps steps of every
 // population in one launch, ny <= kFreeRows, FP64 or FP32 storage.
-constexpr int kFreeSteps = 32, kFreeRows = 4;
-cudaError_t launch_free(bool fp64, int N, int npop, int nsteps, cudaStream_t st, const KernelArgs &a);
+// Populations first .. first + count - 1, count <= kFreePops.
+constexpr int kFreeSteps = 32, kFreeRows = 4, kFreePops = 65535;
+cudaError_t launch_free(bool fp64, int N, int first, int count, int nsteps, cudaStream_t st, const KernelArgs &a);
 
 // Batched persistent form (rlbm_batch.cuh).
 constexpr int kBatchWarps = 6;

@@ -25,12 +25,12 @@ __device__ __forceinline__ float free_lerp(float a, float to, float from) { retu
 __device__ __forceinline__ double free_lerp(double a, double to, double from) { return __fma_rn(a, __dsub_rn(to, from), from); }
 
 template <class T, int NY>
-__global__ void __launch_bounds__(32 * kFreeWarps) rlbm_free_kernel(const KernelArgs a, int N, int nsteps)
+__global__ void __launch_bounds__(32 * kFreeWarps) rlbm_free_kernel(const KernelArgs a, int N, int pop0, int nsteps)
 {
     constexpr int C = kFreeCells / 32, PAD = kFreeCells + kFreeCells / 32;
     __shared__ T buf[kFreeWarps][NY * PAD];
     const int lane = threadIdx.x, w = threadIdx.y;
-    const int i = blockIdx.y; // population
+    const int i = pop0 + blockIdx.y; // population
     const int width = kFreeCells - nsteps, seg = blockIdx.x * kFreeWarps + w;
     if (seg * width >= a.nx) return; // whole warp
     const T *tab = reinterpret_cast<const T *>(a.poptab) + size_t(i) * tab_width(N);
@@ -94,10 +94,11 @@ __global__ void __launch_bounds__(32 * kFreeWarps) rlbm_free_kernel(const Kernel
         }
 }
 
-cudaError_t launch_free(bool fp64, int N, int npop, int nsteps, cudaStream_t st, const KernelArgs &a)
+cudaError_t launch_free(bool fp64, int N, int first, int count, int nsteps, cudaStream_t st, const KernelArgs &a)
 {
-    if (nsteps < 1 || nsteps > kFreeSteps || a.ny < 1 || a.ny > kFreeRows) return cudaErrorInvalidValue;
-    void (*k)(const KernelArgs, int, int) = nullptr;
+    if (nsteps < 1 || nsteps > kFreeSteps || a.ny < 1 || a.ny > kFreeRows || count < 1 || count > kFreePops)
+        return cudaErrorInvalidValue;
+    void (*k)(const KernelArgs, int, int, int) = nullptr;
     switch (a.ny) {
     case 1: k = fp64 ? rlbm_free_kernel<double, 1> : rlbm_free_kernel<float, 1>; break;
     case 2: k = fp64 ? rlbm_free_kernel<double, 2> : rlbm_free_kernel<float, 2>; break;
@@ -105,7 +106,7 @@ cudaError_t launch_free(bool fp64, int N, int npop, int nsteps, cudaStream_t st,
     default: k = fp64 ? rlbm_free_kernel<double, 4> : rlbm_free_kernel<float, 4>; break;
     }
     const int width = kFreeCells - nsteps, segs = (a.nx + width - 1) / width;
-    k<<<dim3((segs + kFreeWarps - 1) / kFreeWarps, npop), dim3(32, kFreeWarps), 0, st>>>(a, N, nsteps);
+    k<<<dim3((segs + kFreeWarps - 1) / kFreeWarps, count), dim3(32, kFreeWarps), 0, st>>>(a, N, first, nsteps);
     return cudaGetLastError();
 }
 

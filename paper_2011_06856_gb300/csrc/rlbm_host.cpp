@@ -893,6 +893,22 @@ cudaError_t launch_step(rlbm_t *h, int from)
     return launch(h, rlbmk::MODE_STEP, a);
 }
 
+// nsteps <= kFreeSteps steps of free streaming on a thin grid; a launch takes kFreePops
+// populations (its grid's y dimension holds 65535).
+cudaError_t launch_free_steps(rlbm_t *h, int nsteps)
+{
+    rlbmk::KernelArgs a = h->base;
+    a.fin = buffer(h, h->cur);
+    a.fout = buffer(h, 1 - h->cur);
+    for (int first = 0; first < h->npop; first += rlbmk::kFreePops) {
+        cudaError_t e = rlbmk::launch_free(h->prec == RLBM_FP64, h->N, first, std::min(h->npop - first, rlbmk::kFreePops),
+                                           nsteps, h->stream, a);
+        if (e != cudaSuccess) return e;
+        ++h->launches;
+    }
+    return cudaSuccess;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -1453,12 +1469,8 @@ rlbm_status rlbm_step(rlbm_t *h, int nsteps)
                            !h->q.onlat && !h->stall_next;
     while (free_thin && left > 0) {
         const int n = std::min(left, rlbmk::kFreeSteps);
-        rlbmk::KernelArgs a = h->base;
-        a.fin = buffer(h, h->cur);
-        a.fout = buffer(h, 1 - h->cur);
-        cudaError_t e = rlbmk::launch_free(h->prec == RLBM_FP64, h->N, h->npop, n, h->stream, a);
+        cudaError_t e = launch_free_steps(h, n);
         if (e != cudaSuccess) return cuda_fail(h, e, "free-streaming kernel");
-        ++h->launches;
         h->cur = 1 - h->cur;
         h->steps += n;
         left -= n;

@@ -909,6 +909,16 @@ cudaError_t launch_free_steps(rlbm_t *h, int nsteps)
     return cudaSuccess;
 }
 
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -1467,13 +1477,20 @@ rlbm_status rlbm_step(rlbm_t *h, int nsteps)
     // of more rows, 16-bit storage and the on-lattice shifts step one launch at a time
     const bool free_thin = std::isinf(h->tau) && h->grid.ny <= rlbmk::kFreeRows && storage_size(h->prec) >= 4 &&
                            !h->q.onlat && !h->stall_next;
-    while (free_thin && left > 0) {
-        const int n = std::min(left, rlbmk::kFreeSteps);
-        cudaError_t e = launch_free_steps(h, n);
-        if (e != cudaSuccess) return cuda_fail(h, e, "free-streaming kernel");
-        h->cur = 1 - h->cur;
-        h->steps += n;
-        left -= n;
+    if (free_thin && left > 0) {
+        // Launches of equal length.  A captured launch is replayed on the buffers of its
+        // capture: there the launches change buffers as often as the steps would, so that an
+        // even number of steps returns to its input and a replay goes on from it.
+        int n = (left + rlbmk::kFreeSteps - 1) / rlbmk::kFreeSteps;
+        if (((n ^ left) & 1) && capturing(h->stream)) ++n;
+        for (; n > 0; --n) {
+            const int steps = (left + n - 1) / n;
+            cudaError_t e = launch_free_steps(h, steps);
+            if (e != cudaSuccess) return cuda_fail(h, e, "free-streaming kernel");
+            h->cur = 1 - h->cur;
+            h->steps += steps;
+            left -= steps;
+        }
     }
     while (left >= kGraphSteps) {
         rlbm_status st = ensure_graph(h, h->cur);

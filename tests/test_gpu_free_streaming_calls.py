@@ -43,3 +43,24 @@ def test_more_populations_than_a_grid_dimension(K, precision):
         sim.sync()
         got = sim.get_populations()[:, 0, :].astype(np.float64)
     assert np.max(np.abs(got - ref)) < (1e-12 if precision == "fp64" else 6 * steps * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("nsteps", [2, 6, 30, 32, 64, 96])
+def test_captured_steps_go_on_at_every_replay(nsteps):
+    """An even number of steps captured on the handle's stream ends in the buffer it started
+    from: each replay advances the state by nsteps, bit for bit as plain steps do."""
+    nx, ny, N, K, replays = 300, 2, 2, 12, 3
+    f0 = W.random_populations(K * (N + 1), ny, nx, seed=nsteps).astype(np.float32)
+    with R.Simulation(nx, ny, N, K, math.inf, "fp32", PER, OUT) as ref:
+        ref.set_populations(f0)
+        ref.step(replays * nsteps)
+        want = ref.get_populations()
+    with R.Simulation(nx, ny, N, K, math.inf, "fp32", PER, OUT) as sim:
+        sim.set_populations(f0)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=sim.stream):
+            sim.step(nsteps)
+        for _ in range(replays):
+            graph.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(sim.get_populations(), want)

@@ -278,9 +278,11 @@ int rlbm_population_groups(const rlbm_t *h);
  * handle's own problem, launches_per_trial launches each, and keep the
  * fastest.  The populations of the current state are not modified (trials
  * read the current buffer and write the other one).  Results are cached per
- * (grid, N, K, precision, boundary conditions) for the life of the process.
- * best_ms (may be NULL) receives the time of one step launch with the chosen
- * tiling.  Synchronises the stream. */
+ * (grid, N, K, precision, boundary conditions, statistic, on- or off-lattice
+ * rule, finite or infinite tau) for the life of the process.  best_ms (may be
+ * NULL) receives the time of one step launch with the chosen tiling (a free
+ * streaming of several steps on up to four rows does not run that kernel, see
+ * rlbm_step).  Synchronises the stream. */
 rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms);
 
 /* Bound, in SM clock cycles, of every mbarrier wait in the TMA-staged, the

@@ -1197,8 +1197,10 @@ int kernel_kind(const rlbm_t *h)
     return h->use_tma ? 1 : 0;
 }
 
+// form: bits for the FP64 per-site part, the on-lattice rule, the statistic and free streaming
+// (its steps do no collision and have two of the kernels to choose from).
 struct TuneKey {
-    int nx, ny, N, K, prec, bcx, bcy, site64;
+    int nx, ny, N, K, prec, bcx, bcy, form;
     bool operator<(const TuneKey &o) const
     {
         return std::memcmp(this, &o, sizeof(TuneKey)) < 0;
@@ -1641,7 +1643,8 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
     if (!h) return fail(nullptr, RLBM_ERR_ARG, "NULL handle");
     if (launches_per_trial < 1) return fail(h, RLBM_ERR_ARG, "launches_per_trial must be >= 1");
     const TuneKey key{h->grid.nx, h->grid.ny, h->N, h->K, h->prec, h->grid.bc_x, h->grid.bc_y,
-                      (h->site_fp64 ? 1 : 0) | (h->q.onlat ? 2 : 0) | (h->stat ? (h->stat > 0 ? 4 : 8) : 0)};
+                      (h->site_fp64 ? 1 : 0) | (h->q.onlat ? 2 : 0) | (h->stat ? (h->stat > 0 ? 4 : 8) : 0) |
+                          (std::isinf(h->tau) ? 16 : 0)};
     {
         std::lock_guard<std::mutex> lk(g_tune_mutex);
         auto it = tune_cache().find(key);

@@ -286,15 +286,17 @@ int rlbm_population_groups(const rlbm_t *h);
 rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms);
 
 /* Bound, in SM clock cycles, of every mbarrier wait in the TMA-staged, the
- * tile-staged and the bulk-staged step kernels (default 4e9, about 2 s).  A wait that runs out
- * makes the kernel record RLBM_ERR_TIMEOUT, drain its own copies (bounded) and
- * skip its stores; the next synchronising call reports it.  cycles >= 1000. */
+ * tile-staged and the bulk-staged step kernels and of the two-pass kernel's waits
+ * on its counters (default 4e9, about 2 s).  A wait that runs out makes the kernel
+ * record RLBM_ERR_TIMEOUT, drain its own copies (bounded) and skip its stores; the
+ * next synchronising call reports it.  cycles >= 1000. */
 rlbm_status rlbm_set_wait_limit(rlbm_t *h, long long cycles);
 
-/* Test hook for the timeout path: the next step launch expects 16 bytes more
- * than its copies deliver, so its waits run out after the wait limit.
- * RLBM_ERR_UNSUPPORTED when the step kernel has no device waits (per-tile,
- * two sites per lane without staging). */
+/* Test hook for the timeout path: the next step launch expects more than
+ * arrives (16 bytes beyond its copies, or in the two-pass kernel more CTAs than
+ * the tile has), so its waits run out after the wait limit.
+ * RLBM_ERR_UNSUPPORTED when the step kernel has no device waits (per-tile, two
+ * sites per lane without staging). */
 rlbm_status rlbm_test_stall_next_step(rlbm_t *h);
 
 /* ------------------------------------------------------------------ */

@@ -799,6 +799,13 @@ cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
     return e;
 }
 
+// The handle's step is the two-pass kernel (launch_step, launch_pair).
+bool runs_split(const rlbm_t *h)
+{
+    if (!h->d_split || h->use_tma || h->use_pair_tma) return false;
+    return h->use_pair ? h->pair_bulk || h->R > 1 : !quad_possible(h, h->P);
+}
+
 cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
     if (!h->pair_bulk && h->R == 1) return launch_quad(h, rlbmk::kMapRow, a);
@@ -881,11 +888,9 @@ cudaError_t launch_step(rlbm_t *h, int from)
     rlbmk::KernelArgs a = h->base;
     a.fin = buffer(h, from);
     a.fout = buffer(h, 1 - from);
-    if (h->use_pair) {
-        if (h->pair_bulk && h->stall_next) a.extra_tx = 16u;
-        h->stall_next = false;
-        return launch_pair(h, a);
-    }
+    if ((h->pair_bulk || runs_split(h)) && h->stall_next) a.extra_tx = 16u;
+    h->stall_next = false;
+    if (h->use_pair) return launch_pair(h, a);
     const int map = h->grid.ny > 1 ? rlbmk::kMapCol : rlbmk::kMapSplit; // for any nx
     if (quad_possible(h, h->P)) return launch_quad(h, map, a);
     if (h->d_split) return launch_split(h, map, a);
@@ -1718,7 +1723,7 @@ rlbm_status rlbm_set_wait_limit(rlbm_t *h, long long cycles)
 rlbm_status rlbm_test_stall_next_step(rlbm_t *h)
 {
     if (!h) return fail(nullptr, RLBM_ERR_ARG, "NULL handle");
-    if (!h->use_tma && !h->pair_bulk && !h->use_pair_tma)
+    if (!h->use_tma && !h->pair_bulk && !h->use_pair_tma && !runs_split(h))
         return fail(h, RLBM_ERR_UNSUPPORTED, "this step kernel has no device waits");
     h->stall_next = true;
     return RLBM_OK;

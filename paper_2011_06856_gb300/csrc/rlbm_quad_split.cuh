@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
                 p.template load<1>(b[1], j * Sb, KS);
             };
             load(j0); // before the wait
-            if (first) s_last = split_wait(a, word, base, unsigned(PARTS + 1)) ? 0u : 2u;
+            if (first) s_last = split_wait(a, word, base, unsigned(PARTS + 1) + (a.extra_tx << 16)) ? 0u : 2u;
             __syncthreads();
             if (s_last) return;
             float2 cf[NC], o[3];

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(128) apply_kernel(Net net, CoarseTab q, float 
 //   y' = Q y = h2 (W3 Q^T) + Q b3: W3' = W3 - (W3 V^T) U^T with V = C W and U = C^T A^-1
 //   (FP32) is kept as a BF16 pair hi + lo (relative error 2^-17), so that C W y' vanishes to
 //   FP32 rounding.  The update is then f += n0 w_i y'_i.  The weights are laid out for the
-//   kernel's shared memory whenever they change (fold_kernel); each CTA only copies them.
+//   kernel's shared memory whenever they change (refresh_kernel); each CTA only copies them.
 // * Features.  Lane (site, half) loads half of every shell's angles into registers, sums
 //   them (per-shell angular sums S0, Sc, Ss, Scc, Scs, Sss folded with p_r, p_r^2), the
 //   halves are joined by a shuffle, and the lane writes its populations / (w_i n0) as BF16
@@ -553,7 +553,7 @@ struct TcGeom {
     static constexpr int SX = 16 * KS1 + 8;   // input row stride: odd number of 16-byte units
     static constexpr int NT3 = NPOP / 8;      // n-tiles of layer 3
     static constexpr int LY = NPOP + 2;       // row stride of y': 64-bit reads of 16 rows without bank conflicts
-    // the prepared weights and tables (fold_kernel), copied to the start of shared memory
+    // the prepared weights and tables (refresh_kernel), copied to the start of shared memory
     static constexpr size_t W1 = 0, W2 = W1 + size_t(64) * SX * 2, W3H = W2 + size_t(64) * SH * 2,
                             W3L = W3H + size_t(NPOP) * SH * 2, BIAS = W3L + size_t(NPOP) * SH * 2,
                             TAB = BIAS + size_t(128 + NPOP) * 4, // b1 b2 b3' | v_x, v_y, 1 / w, w per population, p_r
@@ -562,68 +562,6 @@ struct TcGeom {
                             WARP = ((XA > YS ? XA : YS) + 15) / 16 * 16, TOTAL = FOLD + TC_WARPS * WARP;
 };
 constexpr size_t kFoldMaxBytes = 128 * 1024;
-
-// The BF16 weights, the folded last layer and the tables in the layout of apply_tc_kernel's
-// shared memory; one thread per element, the projections (W3 V^T)[64][4], (V b3)[4] once per CTA.
-template <int N, int K>
-__global__ void __launch_bounds__(256) fold_kernel(Net net, CoarseTab q, unsigned char *fold)
-{
-    using Gm = TcGeom<N, K>;
-    constexpr int NPOP = Gm::NPOP, F = Gm::F, SX = Gm::SX;
-    static_assert(Gm::FOLD <= kFoldMaxBytes, "fold buffer");
-    __shared__ float cm[4][NPOP], wv[65 * 4];
-    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W1);
-    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W2);
-    __nv_bfloat16 *w3h = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W3H);
-    __nv_bfloat16 *w3l = reinterpret_cast<__nv_bfloat16 *>(fold + Gm::W3L);
-    float *bias = reinterpret_cast<float *>(fold + Gm::BIAS), *tab = reinterpret_cast<float *>(fold + Gm::TAB);
-    // C[a][j] for a = 0..3: p, p^2, p^2 c, p^2 s
-    for (int j = threadIdx.x; j < NPOP; j += blockDim.x) {
-        const float p = q.p0[j];
-        cm[0][j] = p;
-        cm[1][j] = p * p;
-        cm[2][j] = p * p * q.c[j];
-        cm[3][j] = p * p * q.s[j];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 65 * 4; e += blockDim.x) {
-        const int k = e >> 2, a = e & 3;
-        float acc = 0.f;
-#pragma unroll 8
-        for (int j = 0; j < NPOP; ++j) acc += (k < 64 ? __bfloat162float(net.W3[k * NPOP + j]) : net.b3[j]) * cm[a][j] * q.w[j];
-        wv[e] = acc;
-    }
-    __syncthreads();
-    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    for (int e = t0; e < 64 * SX; e += nt) w1t[e] = e % SX < F ? net.W1[(e % SX) * H + e / SX] : zero;
-    for (int e = t0; e < 64 * SH; e += nt) w2t[e] = e % SH < H ? net.W2[(e % SH) * H + e / SH] : zero;
-    // W3'[k][i] = W3[k][i] - sum_a (W3 V^T)[k][a] U[i][a], U = C^T A^-1; b3' likewise (k = 64)
-    for (int e = t0; e < NPOP * SH; e += nt) {
-        const int i = e / SH, k = e % SH;
-        float v = 0.f;
-        if (k <= H) {
-            v = k < H ? __bfloat162float(net.W3[k * NPOP + i]) : net.b3[i];
-            float d = 0.f;
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-                d += wv[k * 4 + a] * (cm[0][i] * q.Ainv[a] + cm[1][i] * q.Ainv[4 + a] + cm[2][i] * q.Ainv[8 + a] + cm[3][i] * q.Ainv[12 + a]);
-            v -= d;
-        }
-        if (k == H) bias[128 + i] = v;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(k < H ? v : 0.f);
-        w3h[e] = hi;
-        w3l[e] = __float2bfloat16_rn(k < H ? v - __bfloat162float(hi) : 0.f);
-    }
-    for (int e = t0; e < 128; e += nt) bias[e] = e < 64 ? net.b1[e] : net.b2[e - 64];
-    for (int e = t0; e < NPOP; e += nt) {
-        tab[e] = q.c[e];
-        tab[NPOP + e] = q.s[e];
-        tab[2 * NPOP + e] = 1.f / q.w[e];
-        tab[3 * NPOP + e] = q.w[e];
-    }
-    for (int e = t0; e < 8; e += nt) tab[4 * NPOP + e] = e <= N ? q.p0[e * K] : 0.f;
-}
 
 template <int N, int K>
 __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsigned char *__restrict__ fold, float *__restrict__ f,
@@ -758,7 +696,6 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) apply_tc_kernel(const unsign
 }
 
 using TcKernel = void (*)(const unsigned char *, float *, long long, float);
-using FoldKernel = void (*)(Net, CoarseTab, unsigned char *);
 
 // the specialisations: (N, K) with N_pop a multiple of 8 and at most 80 outputs
 TcKernel tc_kernel(int N, int K, size_t *smem)
@@ -766,13 +703,6 @@ TcKernel tc_kernel(int N, int K, size_t *smem)
     if (N == 2 && K == 24) { *smem = TcGeom<2, 24>::TOTAL; return apply_tc_kernel<2, 24>; }
     if (N == 2 && K == 16) { *smem = TcGeom<2, 16>::TOTAL; return apply_tc_kernel<2, 16>; }
     if (N == 3 && K == 16) { *smem = TcGeom<3, 16>::TOTAL; return apply_tc_kernel<3, 16>; }
-    return nullptr;
-}
-FoldKernel fold_kernel_of(int N, int K)
-{
-    if (N == 2 && K == 24) return fold_kernel<2, 24>;
-    if (N == 2 && K == 16) return fold_kernel<2, 16>;
-    if (N == 3 && K == 16) return fold_kernel<3, 16>;
     return nullptr;
 }
 
@@ -830,7 +760,7 @@ struct TrGeom {
     // strips of the weight gradients: 4 x 2 of gW3 (NT3 / 2 column tiles, the second one more
     // if odd), 4 x 2 of gW2, KS1 x 2 of gW1 (4 column tiles); a warp's blocks
     static constexpr int NS = 16 + 2 * KS1, NSW = (NS + TR_WARPS - 1) / TR_WARPS, NTS = (NT3 + 1) / 2 > 4 ? (NT3 + 1) / 2 : 4;
-    // W1^T and W2^T as in TcGeom, then (fold_kernel, from PREP in its buffer) W2, W3^T, W3, b1 b2 b3
+    // W1^T and W2^T as in TcGeom, then (refresh_kernel, from PREP in its buffer) W2, W3^T, W3, b1 b2 b3
     static constexpr size_t W1T = 0, W2T = W1T + size_t(64) * SX * 2, W2N = W2T + size_t(64) * SH * 2,
                             W3T = W2N + size_t(64) * SH * 2, W3N = W3T + size_t(O) * SH * 2,
                             BIAS = W3N + size_t(64) * SO * 2, XA = (BIAS + size_t(128 + OP) * 4 + 15) / 16 * 16,
@@ -843,24 +773,101 @@ struct TrGeom {
     static_assert(PREP_END <= kFoldMaxBytes, "fold buffer");
 };
 
-// The training kernel's copies of the weights, after apply_tc_kernel's (fold_kernel).
+// The weights as the kernels read them, from the FP32 master: BF16 (w), and in fold the BF16
+// weights, the folded last layer and the tables in the layout of apply_tc_kernel's shared
+// memory, then the training kernel's copies.  One launch per change of the parameters (three
+// dependent ones, one per form, took 15 us more of a 22 us rlbm_closure_set_params).  The first
+// FOLD_CTAS CTAs form W3' (each stages W3 and forms the projections (W3 V^T)[64][4], (V b3)[4]),
+// the others copy.
+struct Master {
+    const float *W1, *W2, *W3, *b1, *b2, *b3;
+};
+constexpr int FOLD_CTAS = 8, COPY_CTAS = 40;
+
 template <int N, int K>
-__global__ void __launch_bounds__(256) prep_kernel(Net net, unsigned char *fold)
+__global__ void __launch_bounds__(256) refresh_kernel(Master net, CoarseTab q, const float *__restrict__ p,
+                                                      const int *__restrict__ map, int nw, __nv_bfloat16 *__restrict__ w,
+                                                      unsigned char *__restrict__ fold)
 {
-    using Gm = TrGeom<N, K>;
-    constexpr int O = Gm::O, SO = Gm::SO, OP = Gm::OP;
-    unsigned char *p = fold + Gm::PREP;
-    __nv_bfloat16 *w2n = reinterpret_cast<__nv_bfloat16 *>(p);
-    __nv_bfloat16 *w3t = reinterpret_cast<__nv_bfloat16 *>(p + (Gm::W3T - Gm::W2N));
-    __nv_bfloat16 *w3n = reinterpret_cast<__nv_bfloat16 *>(p + (Gm::W3N - Gm::W2N));
-    float *bias = reinterpret_cast<float *>(p + (Gm::BIAS - Gm::W2N));
-    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    for (int e = t0; e < 64 * SH; e += nt) w2n[e] = e % SH < H ? net.W2[(e / SH) * H + e % SH] : zero;
-    for (int e = t0; e < O * SH; e += nt) w3t[e] = e % SH < H ? net.W3[(e % SH) * O + e / SH] : zero;
-    for (int e = t0; e < 64 * SO; e += nt) w3n[e] = e % SO < O ? net.W3[(e / SO) * O + e % SO] : zero;
-    for (int e = t0; e < 128 + OP; e += nt)
-        bias[e] = e < 64 ? net.b1[e] : e < 128 ? net.b2[e - 64] : (e - 128 < O ? net.b3[e - 128] : 0.f);
+    using Tc = TcGeom<N, K>;
+    using Tr = TrGeom<N, K>;
+    constexpr int NPOP = Tc::NPOP, F = Tc::F, SX = Tc::SX, SO = Tr::SO, OP = Tr::OP;
+    static_assert(Tc::FOLD <= kFoldMaxBytes, "fold buffer");
+    float *bias = reinterpret_cast<float *>(fold + Tc::BIAS), *tab = reinterpret_cast<float *>(fold + Tc::TAB);
+    const int tid = threadIdx.x;
+    if (blockIdx.x < FOLD_CTAS) {
+        __shared__ float w3[65 * NPOP], cm[4][NPOP], wq[NPOP], wv[65 * 4];
+        // C[a][j] for a = 0..3: p, p^2, p^2 c, p^2 s
+        for (int j = tid; j < NPOP; j += 256) {
+            const float pj = q.p0[j];
+            cm[0][j] = pj;
+            cm[1][j] = pj * pj;
+            cm[2][j] = pj * pj * q.c[j];
+            cm[3][j] = pj * pj * q.s[j];
+            wq[j] = q.w[j];
+        }
+#pragma unroll 4
+        for (int e = tid; e < 65 * NPOP; e += 256)
+            w3[e] = e < 64 * NPOP ? __bfloat162float(__float2bfloat16_rn(net.W3[e])) : net.b3[e - 64 * NPOP];
+        __syncthreads();
+        for (int e = tid; e < 65 * 4; e += 256) {
+            const int k = e >> 2, a = e & 3;
+            float acc = 0.f;
+#pragma unroll 8
+            for (int j = 0; j < NPOP; ++j) acc += w3[k * NPOP + j] * cm[a][j] * wq[j];
+            wv[e] = acc;
+        }
+        __syncthreads();
+        // W3'[k][i] = W3[k][i] - sum_a (W3 V^T)[k][a] U[i][a], U = C^T A^-1; b3' likewise (k = 64)
+        __nv_bfloat16 *w3h = reinterpret_cast<__nv_bfloat16 *>(fold + Tc::W3H);
+        __nv_bfloat16 *w3l = reinterpret_cast<__nv_bfloat16 *>(fold + Tc::W3L);
+        for (int e = blockIdx.x * 256 + tid; e < NPOP * SH; e += FOLD_CTAS * 256) {
+            const int i = e / SH, k = e % SH;
+            float v = 0.f;
+            if (k <= H) {
+                v = w3[k * NPOP + i];
+                float d = 0.f;
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    d += wv[k * 4 + a] * (cm[0][i] * q.Ainv[a] + cm[1][i] * q.Ainv[4 + a] + cm[2][i] * q.Ainv[8 + a] + cm[3][i] * q.Ainv[12 + a]);
+                v -= d;
+            }
+            if (k == H) bias[128 + i] = v;
+            const __nv_bfloat16 hi = __float2bfloat16_rn(k < H ? v : 0.f);
+            w3h[e] = hi;
+            w3l[e] = __float2bfloat16_rn(k < H ? v - __bfloat162float(hi) : 0.f);
+        }
+        return;
+    }
+    unsigned char *prep = fold + Tr::PREP;
+    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(fold + Tc::W1);
+    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(fold + Tc::W2);
+    __nv_bfloat16 *w2n = reinterpret_cast<__nv_bfloat16 *>(prep);
+    __nv_bfloat16 *w3t = reinterpret_cast<__nv_bfloat16 *>(prep + (Tr::W3T - Tr::W2N));
+    __nv_bfloat16 *w3n = reinterpret_cast<__nv_bfloat16 *>(prep + (Tr::W3N - Tr::W2N));
+    float *tbias = reinterpret_cast<float *>(prep + (Tr::BIAS - Tr::W2N));
+    const int t0 = (blockIdx.x - FOLD_CTAS) * 256 + tid, nt = COPY_CTAS * 256;
+    auto bf = [](bool in, const float *v) { return __float2bfloat16_rn(in ? *v : 0.f); };
+    for (int e = t0; e < nw; e += nt) w[e] = __float2bfloat16_rn(p[map[e]]);
+    for (int e = t0; e < 64 * SX; e += nt) w1t[e] = bf(e % SX < F, net.W1 + (e % SX) * H + e / SX);
+    for (int e = t0; e < 64 * SH; e += nt) {
+        w2t[e] = bf(e % SH < H, net.W2 + (e % SH) * H + e / SH);
+        w2n[e] = bf(e % SH < H, net.W2 + (e / SH) * H + e % SH);
+    }
+    for (int e = t0; e < NPOP * SH; e += nt) w3t[e] = bf(e % SH < H, net.W3 + (e % SH) * NPOP + e / SH);
+    for (int e = t0; e < 64 * SO; e += nt) w3n[e] = bf(e % SO < NPOP, net.W3 + (e / SO) * NPOP + e % SO);
+    for (int e = t0; e < 128 + OP; e += nt) {
+        const float b = e < 64 ? net.b1[e] : e < 128 ? net.b2[e - 64] : (e - 128 < NPOP ? net.b3[e - 128] : 0.f);
+        tbias[e] = b;
+        if (e < 128) bias[e] = b;
+    }
+    for (int e = t0; e < NPOP; e += nt) {
+        tab[e] = q.c[e];
+        tab[NPOP + e] = q.s[e];
+        tab[2 * NPOP + e] = 1.f / q.w[e];
+        tab[3 * NPOP + e] = q.w[e];
+    }
+    for (int e = t0; e < 8; e += nt) tab[4 * NPOP + e] = e <= N ? q.p0[e * K] : 0.f;
 }
 
 // GELU of two values (as gelu2) and its derivative Phi(x) + x exp(-x^2 / 2) / sqrt(2 pi)
@@ -1172,7 +1179,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32, 1)
 }
 
 using TrKernel = void (*)(const unsigned char *, const float *, const float *, long long, long long, int, float, float *, float *);
-using PrepKernel = void (*)(Net, unsigned char *);
+using RefreshKernel = void (*)(Master, CoarseTab, const float *, const int *, int, __nv_bfloat16 *, unsigned char *);
 
 TrKernel tr_kernel(int N, int K, size_t *smem)
 {
@@ -1181,11 +1188,11 @@ TrKernel tr_kernel(int N, int K, size_t *smem)
     if (N == 3 && K == 16) { *smem = TrGeom<3, 16>::TOTAL; return train_tc_kernel<3, 16>; }
     return nullptr;
 }
-PrepKernel prep_kernel_of(int N, int K)
+RefreshKernel refresh_kernel_of(int N, int K)
 {
-    if (N == 2 && K == 24) return prep_kernel<2, 24>;
-    if (N == 2 && K == 16) return prep_kernel<2, 16>;
-    if (N == 3 && K == 16) return prep_kernel<3, 16>;
+    if (N == 2 && K == 24) return refresh_kernel<2, 24>;
+    if (N == 2 && K == 16) return refresh_kernel<2, 16>;
+    if (N == 3 && K == 16) return refresh_kernel<3, 16>;
     return nullptr;
 }
 
@@ -1283,13 +1290,14 @@ bool tc_attributes(const rlbm_closure *c)
 rlbm_status refresh_bf16(rlbm_closure *c)
 {
     const int nw = c->F * H + H * H + H * c->O;
-    to_bf16_kernel<<<(nw + 255) / 256, 256, 0, c->stream>>>(c->d_p, c->d_w, c->d_wmap, nw);
-    CL_CUDA(c, cudaGetLastError());
-    if (FoldKernel k = fold_kernel_of(c->N, c->K)) { // in stream order, also under capture
-        k<<<16, 256, 0, c->stream>>>(net_of(c), tab_of(c), c->d_fold);
-        prep_kernel_of(c->N, c->K)<<<16, 256, 0, c->stream>>>(net_of(c), c->d_fold);
-        CL_CUDA(c, cudaGetLastError());
+    if (RefreshKernel k = refresh_kernel_of(c->N, c->K)) { // in stream order, also under capture
+        const float *p = c->d_p;
+        const Master net{p + c->off_W1, p + c->off_W2, p + c->off_W3, p + c->off_b1, p + c->off_b2, p + c->off_b3};
+        k<<<FOLD_CTAS + COPY_CTAS, 256, 0, c->stream>>>(net, tab_of(c), p, c->d_wmap, nw, c->d_w, c->d_fold);
+    } else {
+        to_bf16_kernel<<<(nw + 255) / 256, 256, 0, c->stream>>>(c->d_p, c->d_w, c->d_wmap, nw);
     }
+    CL_CUDA(c, cudaGetLastError());
     return RLBM_OK;
 }
 

@@ -278,9 +278,10 @@ struct rlbm {
     rlbmk::TmaArgs *tma = nullptr; // [2]: input buffer 0 / 1
     int tma_grid = 0;
     size_t tma_smem = 0;
-    int sm_count = 0;
+    int sm_count = 0, max_smem = 0;
     bool stall_next = false; // test hook: next launch waits for bytes that never arrive
     bool no_tma = false;     // tiling choice: per-tile kernel even where TMA is possible
+    bool plain = false;      // kind 0: the per-tile kernel itself, not a quadrant kernel in its place
     bool use_pair = false;   // two-sites-per-lane step kernel (rlbm_pair.cuh)
     bool pair_bulk = false;  // ... with its first pass staged by cp.async.bulk on interior tiles
     bool use_pair_tma = false;          // ... with the whole tile staged by TMA (rlbm_pair_tma.cuh)
@@ -316,6 +317,15 @@ rlbm_status cuda_fail(rlbm_t *h, cudaError_t e, const char *what)
         cudaError_t e_ = (call);                                                                 \
         if (e_ != cudaSuccess) return cuda_fail(h, e_, #call);                                   \
     } while (0)
+
+rlbm_status device_facts(rlbm_t *h)
+{
+    int dev = 0;
+    RLBM_CUDA(h, cudaGetDevice(&dev));
+    RLBM_CUDA(h, cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
+    RLBM_CUDA(h, cudaDeviceGetAttribute(&h->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    return RLBM_OK;
+}
 
 // Pick P (populations per warp, one of the compiled sizes) and Gs (warps per
 // energy shell, G = Gs (N+1) warps per CTA): fewest idle population slots,
@@ -700,14 +710,12 @@ bool quad_possible(const rlbm_t *h, int P)
 // step, per-tile against two passes: ragged tilings (P not dividing K) N = 3, K = 100 292 to
 // 139, K = 84 240 to 129; P = 48 and K = 240 247 to 183.  Fewer than 128 angles in whole
 // warps stay with the per-tile kernel, whose CTAs hold them all (255 x 129, K = 96, P = 48:
-// 59 us, two passes 72), and so do 16-bit grids too small to fill the GPU, whose per-site
-// part is short (999 x 1, N = 3, K = 120: 19.4 us, two passes 21.3).
-constexpr int kSplitMinRaggedK = 64, kSplitMinK = 128, kSplitMinSites16 = 8192;
-bool split_wanted(const rlbm_t *h)
+// 59 us, two passes 72).  Small grids: prefer_plain.
+constexpr int kSplitMinRaggedK = 64, kSplitMinK = 128;
+bool split_possible(const rlbm_t *h)
 {
     return h->prec != RLBM_FP64 && !std::isinf(h->tau) && h->N <= 3 && !h->q.onlat && !h->stat && h->K % 4 == 0 &&
-           h->K >= (h->K % h->P ? kSplitMinRaggedK : kSplitMinK) && !quad_possible(h, h->P) &&
-           (storage_size(h->prec) > 2 || (long long)h->grid.nx * h->grid.ny >= kSplitMinSites16);
+           h->K >= (h->K % h->P ? kSplitMinRaggedK : kSplitMinK) && !quad_possible(h, h->P);
 }
 
 // Its ring and counters for the handle's present tiling (the stream is idle: creation and
@@ -717,12 +725,8 @@ void setup_split(rlbm_t *h)
 {
     if (h->d_split) cudaFree(h->d_split);
     h->d_split = nullptr;
-    if (!split_wanted(h)) return;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return;
-    const int resident = sms * rlbmk::kSplitCtasPerSm;
+    if (h->plain || !split_possible(h)) return;
+    const int resident = h->sm_count * rlbmk::kSplitCtasPerSm;
     const long long tiles = std::max((h->grid.nx + 63ll) / 64 * h->grid.ny, (h->grid.nx + 31ll) / 32 * ((h->grid.ny + 1ll) / 2));
     // one CTA per shell of a tile (a CTA's start and end cost as much as a few quads per
     // warp: 256^2, N = 3, K = 600, one, two, four per shell 487, 514, 602 us); more only
@@ -769,6 +773,33 @@ bool quad64_possible(const rlbm_t *h)
            (P == 8 || P == 12 || P == 16 || P == 24 || P == 32) && h->K % P == 0;
 }
 
+// Kind 0 has one of the quadrant kernels to run in place of the per-tile kernel.
+bool stand_in_possible(const rlbm_t *h) { return quad_possible(h, h->P) || split_possible(h) || quad64_possible(h); }
+
+// Where kind 0 runs the per-tile kernel all the same unless the autotuner finds otherwise:
+// grids of few tiles, where a step is one CTA's latency.  us per step, per-tile against the
+// kernel in its place (graph replays):
+//  - P = 16, capped at 64 registers: 64^2 FP32 N = 2, K = 64 10.3 and 11.9, 8192 x 1 11.1 and
+//    10.0; FP16 8.9 and 10.1, 128 x 96 K = 16 7.7 and 8.5, K = 48 14.9 and 10.7;
+//  - two passes instead of one group of populations per warp: ragged tilings with P <= 32
+//    (64^2 FP32 K = 68, P = 24 14.8 and 21.6, 8192 x 1 22.9 and 20.4), full ones, which idle no
+//    lane (K = 128, P = 64 64^2 17.5 and 24.0, 8192 x 1 17.9 and 24.5, 8191 x 4 87 and 59;
+//    FP16 8192 x 1 15.3 and 24.0, 128^2 32.6 and 36.2, 8191 x 4 67 and 59).
+//    Ragged tilings with P = 48 and 64 idle a third of theirs: two passes on every grid.
+bool prefer_plain(const rlbm_t *h)
+{
+    const long long sites = (long long)h->grid.nx * h->grid.ny;
+    const bool two_bytes = storage_size(h->prec) == 2;
+    if (quad_possible(h, h->P)) {
+        if (h->P != 16 || h->stat) return false;
+        const long long tiles = h->grid.ny > 1 ? (h->grid.nx + 31ll) / 32 * ((h->grid.ny + 1ll) / 2) : (h->grid.nx + 63ll) / 64;
+        return two_bytes ? tiles * h->G < 7ll * h->sm_count : 3 * tiles < 2ll * h->sm_count;
+    }
+    if (!split_possible(h) || h->R > 1) return false;
+    if (h->K % h->P == 0) return sites < (two_bytes ? 24576 : 16384);
+    return two_bytes ? sites < 8192 : h->P <= 32 && sites < 6144;
+}
+
 cudaError_t launch_quad64(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
     const dim3 block(32, h->Gs, h->N + 1);
@@ -803,7 +834,7 @@ cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
 bool runs_split(const rlbm_t *h)
 {
     if (!h->d_split || h->use_tma || h->use_pair_tma) return false;
-    return h->use_pair ? h->pair_bulk || h->R > 1 : !quad_possible(h, h->P);
+    return h->use_pair ? h->pair_bulk || h->R > 1 : !h->plain && !quad_possible(h, h->P);
 }
 
 cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
@@ -892,6 +923,7 @@ cudaError_t launch_step(rlbm_t *h, int from)
     h->stall_next = false;
     if (h->use_pair) return launch_pair(h, a);
     const int map = h->grid.ny > 1 ? rlbmk::kMapCol : rlbmk::kMapSplit; // for any nx
+    if (h->plain) return launch(h, rlbmk::MODE_STEP, a);
     if (quad_possible(h, h->P)) return launch_quad(h, map, a);
     if (h->d_split) return launch_split(h, map, a);
     if (quad64_possible(h)) return launch_quad64(h, a);
@@ -953,11 +985,7 @@ rlbm_status setup_tma(rlbm_t *h)
     const size_t ls = (h->prec == RLBM_FP64 || h->site_fp64) ? 8 : 4;
     const size_t rs = (h->prec == RLBM_FP64) ? 8 : 4;
     const rlbmk::TmaSmem L(stage, h->G, h->P, h->N, rs, ls);
-    int dev = 0, max_smem = 0;
-    RLBM_CUDA(h, cudaGetDevice(&dev));
-    RLBM_CUDA(h, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    RLBM_CUDA(h, cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
-    if (L.total > size_t(max_smem)) return RLBM_OK;
+    if (L.total > size_t(h->max_smem)) return RLBM_OK;
 
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -1058,13 +1086,9 @@ rlbm_status setup_pair_tma(rlbm_t *h)
     const int CB = npop / ncbox;
     if (CB * ncbox != npop || CB % 4 != 0) return RLBM_OK; // whole boxes, 128-byte aligned destinations
     const bool two_d = ny > 1;
-    int dev = 0, max_smem = 0;
-    RLBM_CUDA(h, cudaGetDevice(&dev));
-    RLBM_CUDA(h, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    RLBM_CUDA(h, cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
     const rlbmk::PairTmaSmem L(h->N, h->G, npop, int(es), two_d);
     const size_t need = L.total;
-    if (need > size_t(max_smem)) return RLBM_OK;
+    if (need > size_t(h->max_smem)) return RLBM_OK;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     RLBM_CUDA(h, cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qres));
@@ -1165,7 +1189,10 @@ rlbm_status validate_fields_ptrs(rlbm_t *h, const void *a, const void *b, const 
 
 // Switch the handle to another tiling: P populations per warp and the step
 // kernel kind (0 per-tile, 1 persistent TMA-staged where possible, 2 two
-// sites per lane where possible; otherwise the per-tile kernel).
+// sites per lane where possible; otherwise the per-tile kernel).  Kind 0 leaves
+// it to prefer_plain whether a quadrant kernel takes its place; kKindPlain and
+// kKindStandIn say so (autotuner, batch).
+constexpr int kKindPlain = 5, kKindStandIn = 6;
 rlbm_status retile(rlbm_t *h, int P, int kind)
 {
     RLBM_CUDA(h, cudaStreamSynchronize(h->stream));
@@ -1177,6 +1204,7 @@ rlbm_status retile(rlbm_t *h, int P, int kind)
         h->R = 1;
     }
     h->G = h->Gs * (h->N + 1);
+    h->plain = kind == kKindPlain || (kind == 0 && prefer_plain(h));
     h->no_tma = kind != 1;
     h->use_pair = (kind == 2 || kind == 3 || kind == 4) && pair_possible(h, P);
     h->pair_bulk = h->use_pair && kind == 3 && pair_bulk_possible(h) && h->R == 1;
@@ -1200,6 +1228,13 @@ int kernel_kind(const rlbm_t *h)
     if (h->use_pair_tma) return 4;
     if (h->use_pair) return h->pair_bulk ? 3 : 2;
     return h->use_tma ? 1 : 0;
+}
+
+// The same, kind 0 with a stand-in told apart.
+int tuned_kind(const rlbm_t *h)
+{
+    const int kind = kernel_kind(h);
+    return kind == 0 && stand_in_possible(h) ? (h->plain ? kKindPlain : kKindStandIn) : kind;
 }
 
 // form: bits for the FP64 per-site part, the on-lattice rule, the statistic and free streaming
@@ -1332,9 +1367,13 @@ static rlbm_status create_impl(rlbm_t **out, rlbm_grid grid, int order_N, int an
             else h->own_buf = true;
         }
     }
+    if (st == RLBM_OK) st = device_facts(h);
     if (st == RLBM_OK) st = build_tables(h);
     if (st == RLBM_OK) st = setup_tma(h);
-    if (st == RLBM_OK) setup_split(h);
+    if (st == RLBM_OK) {
+        h->plain = prefer_plain(h);
+        setup_split(h);
+    }
     if (st != RLBM_OK) {
         g_create_error = h->err;
         rlbm_destroy(h);
@@ -1655,7 +1694,7 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
         auto it = tune_cache().find(key);
         if (it != tune_cache().end()) {
             if (best_ms) *best_ms = it->second.ms;
-            if (it->second.P == h->P && it->second.kind == kernel_kind(h)) return RLBM_OK;
+            if (it->second.P == h->P && it->second.kind == tuned_kind(h)) return RLBM_OK;
             return retile(h, it->second.P, it->second.kind);
         }
     }
@@ -1663,7 +1702,7 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
     cudaEvent_t e0, e1;
     RLBM_CUDA(h, cudaEventCreate(&e0));
     RLBM_CUDA(h, cudaEventCreate(&e1));
-    TuneChoice best{h->P, kernel_kind(h), 1e30f};
+    TuneChoice best{h->P, tuned_kind(h), 1e30f};
     const long long launches0 = h->launches;
     rlbm_status st = RLBM_OK;
     for (int P : sizes) {
@@ -1671,10 +1710,10 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
         if (!group_tiling(h->N, h->K, P, gs, ng)) continue;
         if (h->q.onlat && P != 12) continue; // the on-lattice kernel is built for P = 12
         if (P > 2 * h->K) continue;
-        for (int kind = 4; kind >= 0 && st == RLBM_OK; --kind) {
+        for (int kind : {4, 3, 2, 1, kKindStandIn, kKindPlain, 0}) {
             st = retile(h, P, kind);
             if (st) break;
-            if (kernel_kind(h) != kind) continue; // kernel kind not possible for this tiling
+            if (tuned_kind(h) != kind) continue; // kernel kind not possible for this tiling
             // time cur -> other launches (the state in buffer cur is not modified)
             cudaError_t e = launch_step(h, h->cur);
             if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
@@ -1687,6 +1726,7 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
             ms /= launches_per_trial;
             if (ms < best.ms) best = TuneChoice{P, kind, ms};
         }
+        if (st) break;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1921,8 +1961,9 @@ rlbm_status batch_check(rlbm_batch *b)
 constexpr int kBatchStreams = 16;
 
 // Step kernel of a problem in the stream pool at tiling P: two sites per lane, in one
-// row for an even nx, else (kind 0) in the quadrant kernel's forms for any nx.
-int solo_kind_for(const rlbm_t *h, int P) { return pair_possible(h, P) ? 2 : 0; }
+// row for an even nx, else in the quadrant kernel's forms for any nx (the problems together
+// fill the GPU: no per-tile kernel for a small one).
+int solo_kind_for(const rlbm_t *h, int P) { return pair_possible(h, P) ? 2 : quad_possible(h, P) ? kKindStandIn : 0; }
 
 // Smallest two-sites-per-lane tiling of a problem (more, lighter warps per
 // SM), else the per-tile kernel with the default tiling.

@@ -272,8 +272,8 @@ RLBM_DECLARE_QUAD(stat_f32) // the quantum statistics
 RLBM_DECLARE_QUAD(f16)
 RLBM_DECLARE_QUAD(bf16)
 #undef RLBM_DECLARE_QUAD
-cudaError_t launch_quad_f64_n2(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
-cudaError_t launch_quad_f64_n3(int PP, dim3 block, cudaStream_t st, const KernelArgs &a);
+cudaError_t launch_quad_f64_n2(int PP, bool one_row, dim3 block, cudaStream_t st, const KernelArgs &a);
+cudaError_t launch_quad_f64_n3(int PP, bool one_row, dim3 block, cudaStream_t st, const KernelArgs &a);
 // many angles: two passes over the tiles in one launch
 #define RLBM_DECLARE_SPLIT(name)                                                                         \
     cudaError_t launch_split_##name##_n2(int map, bool two_d, cudaStream_t st, const KernelArgs &a);     \

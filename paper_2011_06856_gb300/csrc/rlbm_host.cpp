@@ -803,8 +803,9 @@ bool prefer_plain(const rlbm_t *h)
 cudaError_t launch_quad64(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
     const dim3 block(32, h->Gs, h->N + 1);
-    cudaError_t e = h->N == 2 ? rlbmk::launch_quad_f64_n2(h->P, block, h->stream, a)
-                              : rlbmk::launch_quad_f64_n3(h->P, block, h->stream, a);
+    const bool one_row = (h->grid.nx + 31ll) / 32 * ((h->grid.ny + 1ll) / 2) < h->sm_count;
+    cudaError_t e = h->N == 2 ? rlbmk::launch_quad_f64_n2(h->P, one_row, block, h->stream, a)
+                              : rlbmk::launch_quad_f64_n3(h->P, one_row, block, h->stream, a);
     if (e == cudaSuccess) ++h->launches;
     return e;
 }

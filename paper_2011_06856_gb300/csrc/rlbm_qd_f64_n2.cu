@@ -1,8 +1,8 @@
 // Quadrant step kernel instances: FP64 storage, N = 2.
 #include "rlbm_quad64.cuh"
 namespace rlbmk {
-cudaError_t launch_quad_f64_n2(int PP, dim3 block, cudaStream_t st, const KernelArgs &a)
+cudaError_t launch_quad_f64_n2(int PP, bool one_row, dim3 block, cudaStream_t st, const KernelArgs &a)
 {
-    return launch_quad64_n<2>(PP, block, st, a);
+    return launch_quad64_n<2>(PP, one_row, block, st, a);
 }
 } // namespace rlbmk

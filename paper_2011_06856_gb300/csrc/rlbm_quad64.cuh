@@ -1,6 +1,9 @@
 // Quadrant form of the FP64-storage step (arXiv 2011.06856, Sec. 2.2; N = 2, 3): the
 // populations of a warp in quadruples theta + k pi/2 (rlbm_quad.cuh), one column of the
-// grid per lane, RW = 2 rows of it for ny > 1 (P <= 16) or one.
+// grid per lane, RW = 2 rows of it for ny > 1 (P <= 16) or one.  A grid with fewer tiles of
+// two rows than the GPU has SMs takes one row: the FP64 pipes of twice the SMs share the work
+// (64^2, N = 2, K = 60, P = 12: two rows 59.8 us a step, the per-tile kernel 47.6, one row
+// 35.8).
 //
 // The step is bound by the FP64 pipe (1/64 of the FP32 rate), so what counts is FP64
 // operations per population, N = 3 in 2D: the bilinear pull 5 with two rows per lane (the
@@ -235,17 +238,15 @@ __global__ void __maxnreg__(128) rlbm_quad64_kernel(const KernelArgs a)
 }
 
 template <int N, int PP>
-static cudaError_t launch_quad64_np(dim3 block, cudaStream_t st, const KernelArgs &a)
+static cudaError_t launch_quad64_np(bool one_row, dim3 block, cudaStream_t st, const KernelArgs &a)
 {
-    void (*k)(const KernelArgs);
+    void (*k)(const KernelArgs) = a.ny == 1 ? rlbm_quad64_kernel<N, PP, 1, false> : rlbm_quad64_kernel<N, PP, 1, true>;
     int rw = 1;
-    if (a.ny == 1) {
-        k = rlbm_quad64_kernel<N, PP, 1, false>;
-    } else if constexpr (PP <= 16) {
-        k = rlbm_quad64_kernel<N, PP, 2, true>;
-        rw = 2;
-    } else {
-        k = rlbm_quad64_kernel<N, PP, 1, true>;
+    if constexpr (PP <= 16) {
+        if (a.ny > 1 && !one_row) {
+            k = rlbm_quad64_kernel<N, PP, 2, true>;
+            rw = 2;
+        }
     }
     const int G = int(block.y * block.z), sums = 5 * G, coef = (N + 1) * (2 * N + 1);
     const size_t smem = size_t((sums > coef ? sums : coef) + 8 + (N + 1) * (N + 1) + 3) * 32 * rw * 8;
@@ -258,14 +259,14 @@ static cudaError_t launch_quad64_np(dim3 block, cudaStream_t st, const KernelArg
 }
 
 template <int N>
-static cudaError_t launch_quad64_n(int PP, dim3 block, cudaStream_t st, const KernelArgs &a)
+static cudaError_t launch_quad64_n(int PP, bool one_row, dim3 block, cudaStream_t st, const KernelArgs &a)
 {
     switch (PP) {
-    case 8: return launch_quad64_np<N, 8>(block, st, a);
-    case 12: return launch_quad64_np<N, 12>(block, st, a);
-    case 16: return launch_quad64_np<N, 16>(block, st, a);
-    case 24: return launch_quad64_np<N, 24>(block, st, a);
-    case 32: return launch_quad64_np<N, 32>(block, st, a);
+    case 8: return launch_quad64_np<N, 8>(one_row, block, st, a);
+    case 12: return launch_quad64_np<N, 12>(one_row, block, st, a);
+    case 16: return launch_quad64_np<N, 16>(one_row, block, st, a);
+    case 24: return launch_quad64_np<N, 24>(one_row, block, st, a);
+    case 32: return launch_quad64_np<N, 32>(one_row, block, st, a);
     default: return cudaErrorInvalidValue;
     }
 }

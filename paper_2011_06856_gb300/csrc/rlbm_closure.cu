@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(256) refresh_kernel(Master net, CoarseTab q, c
             cm[3][j] = pj * pj * q.s[j];
             wq[j] = q.w[j];
         }
-#pragma unroll 4
+#pragma unroll
         for (int e = tid; e < 65 * NPOP; e += 256)
             w3[e] = e < 64 * NPOP ? __bfloat162float(__float2bfloat16_rn(net.W3[e])) : net.b3[e - 64 * NPOP];
         __syncthreads();

@@ -28,26 +28,24 @@ RLBM_BITS unsigned rotl32(unsigned x, int n)
 #endif
 }
 
-// The k-th word of a thread is the exclusive or of two hashed words rotated by 5 k and 4 k
-// bits.  Bit i of word k joins bits i - 5 k and i - 4 k of the two, whose distance k comes back
-// after 32 words: up to there no pair of bits meets twice, so that any two bits of the words are
-// independent, which is what the moments of the rounding errors need; word 32 would be word 0
-// again.  (Rotated by 5 k and 3 k, word 16 is word 0 with its halves, the lane's two sites,
-// exchanged.)  A thread that draws more hashes the first of the two again after every kWords
-// words (refresh), 8 integer operations.  A word costs three integer operations on the pipe that
-// the arithmetic leaves idle; an LCG draw (IMAD) takes two cycles of the FMA pipe, a 64-bit
-// product four.
+// The k-th word of a thread is the exclusive or of two hashed words rotated by 5 k and 3 k
+// bits.  Bit i of word k joins bits i - 5 k and i - 3 k of the two, whose distance 2 k comes
+// back after 16 words: up to there no pair of bits meets twice, so that any two bits of the
+// words are independent, which is what the moments of the rounding errors need; word k + 16
+// would be word k with its halves (the lane's two sites) exchanged.  After kWords words the
+// first of the two is therefore hashed again (refresh), 8 integer operations per 16 words.
+// A word costs three integer operations on the pipe that the arithmetic leaves idle; an LCG
+// draw (IMAD) takes two cycles of the FMA pipe, a 64-bit product four.
 struct QuadBits {
-    static constexpr int kWords = 32;
+    static constexpr int kWords = 16;
     unsigned a, b;
     RLBM_BITS unsigned next()
     {
         a = rotl32(a, 5);
-        b = rotl32(b, 4);
+        b = rotl32(b, 3);
         return a ^ b;
     }
-    // (not the constant of quad_seed: the rotations have come round, it would give the second word)
-    RLBM_BITS void refresh() { a = mix32(a + 0x85EBCA6Bu); }
+    RLBM_BITS void refresh() { a = mix32(a + 0x9E3779B9u); }
 };
 
 // Seeded by the thread's first site, the warp g < 256 and the launch counter.  The site is

@@ -48,7 +48,6 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
 {
     constexpr int NC = 2 * N + 1;
     constexpr int QW = PP / 4; // quads per warp
-    static_assert(PP <= QuadBits::kWords, "one word per population");
     constexpr int HX = PairTmaGeom<St>::HX, BW = PairTmaGeom<St>::BW;
     constexpr int RW = TWO_D ? 2 : 1;
     const KernelArgs &a = ta.a;
@@ -175,6 +174,7 @@ __device__ __forceinline__ void pair_tma_body(const PairTmaArgs &ta)
     for (int k = 0; k < QW; ++k) {
         float2 feq[4], om[4];
         quad_equilibrium<N>(cf, o, tb + 3 * k, feq, om);
+        if (k > 0 && 4 * k % QuadBits::kWords == 0) rng.refresh();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             char *p = ob + (k * Sb + u * KS);

@@ -685,7 +685,6 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
 {
     constexpr int NC = 2 * N + 1, QW = PP / 4;
     constexpr bool DD = sizeof(St) == 4;
-    static_assert(PP <= QuadBits::kWords, "one word per population");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x, Gs = blockDim.y, K4 = a.K >> 2;
     const int q = warp_uniform(threadIdx.y), r = warp_uniform(threadIdx.z);
@@ -743,6 +742,7 @@ __global__ void __maxnreg__(PP <= 16 ? 64 : 128) rlbm_quad_kernel(const KernelAr
                               N == 3 ? __ldg(tb + 3 * k + 2) : make_float4(0.f, 0.f, 0.f, 0.f)};
         float2 feq[4], om[4];
         quad_equilibrium<N>(cf, o, tq, feq, om);
+        if (k > 0 && 4 * k % QuadBits::kWords == 0) rng.refresh();
         out.store(k * Sb, KS, fs + 4 * k, feq, om, rng);
     }
     __syncthreads();

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitCtasPerSm) rlbm_quad_s
                 load(j + NW); // its latency passes behind the equilibrium and the stores
                 quad_equilibrium<N>(cf, o, tq, feq, om);
                 out.store(j * Sb, KS, f, feq, om, rng);
-                constexpr int TURN = (QuadBits::kWords / 4 - 1) * NW; // the warp's eighth quad since the last one
+                constexpr int TURN = (QuadBits::kWords / 4 - 1) * NW; // the warp's fourth quad since the last one
                 static_assert((NW & (NW - 1)) == 0, "quads counted by the bits of j - j0");
                 if (((j - j0) & TURN) == TURN) rng.refresh();
             }

@@ -5,7 +5,7 @@ warps), and the seeds of a launch.
 
 Two words of independent bits differ in 16 +- sqrt(8) of their 32 bits.  Over 4096 threads the
 mean is within sqrt(8 / 4096) = 0.044 of 16 (one sigma); 7 sigma are allowed for every pair
-of the first 96 words and every rotation of one against the other, 3e5 means."""
+of the first 48 words and every rotation of one against the other, 7e4 means."""
 import ctypes
 import os
 import shutil
@@ -79,7 +79,7 @@ def test_words_of_a_thread_do_not_repeat(bits, launch):
 
 
 def test_words_of_a_thread_are_uncorrelated(bits):
-    threads, n = 4096, 96
+    threads, n = 4096, 48
     w = draw(bits, range(threads), 5, 3, n)
     d = np.zeros((n, n, 32))
     bits.mean_distance(ctypes.c_void_p(np.ascontiguousarray(w).ctypes.data), threads, n, ctypes.c_void_p(d.ctypes.data))

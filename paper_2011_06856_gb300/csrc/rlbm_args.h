@@ -254,6 +254,18 @@ RLBM_DECLARE_PAIR(f32)
 RLBM_DECLARE_PAIR(f16)
 RLBM_DECLARE_PAIR(bf16)
 #undef RLBM_DECLARE_PAIR
+// several population groups per warp (FP32 storage)
+cudaError_t launch_pair_groups_f32_n2(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                      const KernelArgs &a);
+cudaError_t launch_pair_groups_f32_n3(int PP, bool two_d, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                      const KernelArgs &a);
+inline cudaError_t launch_pair_groups_f32(int N, int PP, bool two_d, dim3 grid, dim3 block, size_t smem,
+                                          cudaStream_t st, const KernelArgs &a)
+{
+    if (N == 2) return launch_pair_groups_f32_n2(PP, two_d, grid, block, smem, st, a);
+    if (N == 3) return launch_pair_groups_f32_n3(PP, two_d, grid, block, smem, st, a);
+    return cudaErrorInvalidValue;
+}
 // Quadrant step kernel (rlbm_quad.cuh); map: QuadMap, how a lane's two sites lie.
 #define RLBM_DECLARE_QUAD(name)                                                                          \
     cudaError_t launch_quad_##name##_n2(int PP, int map, bool two_d, dim3 block, size_t smem,            \

@@ -283,6 +283,7 @@ struct rlbm {
     bool no_tma = false;     // tiling choice: per-tile kernel even where TMA is possible
     bool plain = false;      // kind 0: the per-tile kernel itself, not a quadrant kernel in its place
     bool use_pair = false;   // two-sites-per-lane step kernel (rlbm_pair.cuh)
+    bool groups = false;     // ... several population groups per warp instead of the two-pass kernel
     bool pair_bulk = false;  // ... with its first pass staged by cp.async.bulk on interior tiles
     bool use_pair_tma = false;          // ... with the whole tile staged by TMA (rlbm_pair_tma.cuh)
     rlbmk::PairTmaArgs *ptma = nullptr; // [2]: input buffer 0 / 1
@@ -725,7 +726,7 @@ void setup_split(rlbm_t *h)
 {
     if (h->d_split) cudaFree(h->d_split);
     h->d_split = nullptr;
-    if (h->plain || !split_possible(h)) return;
+    if (h->plain || h->groups || !split_possible(h)) return;
     const int resident = h->sm_count * rlbmk::kSplitCtasPerSm;
     const long long tiles = std::max((h->grid.nx + 63ll) / 64 * h->grid.ny, (h->grid.nx + 31ll) / 32 * ((h->grid.ny + 1ll) / 2));
     // one CTA per shell of a tile (a CTA's start and end cost as much as a few quads per
@@ -835,18 +836,23 @@ cudaError_t launch_quad(rlbm_t *h, int map, const rlbmk::KernelArgs &a)
 bool runs_split(const rlbm_t *h)
 {
     if (!h->d_split || h->use_tma || h->use_pair_tma) return false;
-    return h->use_pair ? h->pair_bulk || h->R > 1 : !h->plain && !quad_possible(h, h->P);
+    return h->use_pair ? h->R > 1 && !h->groups : !h->plain && !quad_possible(h, h->P);
 }
 
 cudaError_t launch_pair(rlbm_t *h, const rlbmk::KernelArgs &a)
 {
     if (!h->pair_bulk && h->R == 1) return launch_quad(h, rlbmk::kMapRow, a);
-    if (h->d_split) return launch_split(h, rlbmk::kMapRow, a);
+    if (runs_split(h)) return launch_split(h, rlbmk::kMapRow, a);
     const dim3 grid((h->grid.nx + rlbmk::kPairSites - 1) / rlbmk::kPairSites, h->grid.ny);
     const dim3 block(32, h->G);
     const bool two_d = h->grid.ny > 1;
-    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, true, int(storage_size(h->prec)), two_d);
+    const size_t smem = rlbmk::pair_smem_total(h->N, h->G, !h->groups, int(storage_size(h->prec)), two_d);
     cudaError_t e;
+    if (h->groups) {
+        e = rlbmk::launch_pair_groups_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a);
+        if (e == cudaSuccess) ++h->launches;
+        return e;
+    }
     switch (h->prec) {
     case RLBM_FP32: e = rlbmk::launch_pair_f32(h->N, h->P, two_d, grid, block, smem, h->stream, a); break;
     case RLBM_FP16_DEV:
@@ -1192,8 +1198,12 @@ rlbm_status validate_fields_ptrs(rlbm_t *h, const void *a, const void *b, const 
 // kernel kind (0 per-tile, 1 persistent TMA-staged where possible, 2 two
 // sites per lane where possible; otherwise the per-tile kernel).  Kind 0 leaves
 // it to prefer_plain whether a quadrant kernel takes its place; kKindPlain and
-// kKindStandIn say so (autotuner, batch).
-constexpr int kKindPlain = 5, kKindStandIn = 6;
+// kKindStandIn say so (autotuner, batch).  Kind 2 with several population groups
+// per warp runs the two-pass kernel; kKindGroups runs the groups, which are the faster
+// ones on some grids of 8 to 16 thousand sites (us a step, groups and two passes:
+// 8192 x 1 N = 2, K = 600, P = 24 46.4 and 66.2, N = 3, K = 288, P = 24 33.5 and 37.4; 128^2 N = 2,
+// K = 400, P = 8 77.0 and 84.7; 96^2 67.0 and 60.8, 32768 x 1 144 and 119): the autotuner tries both.
+constexpr int kKindPlain = 5, kKindStandIn = 6, kKindGroups = 7;
 rlbm_status retile(rlbm_t *h, int P, int kind)
 {
     RLBM_CUDA(h, cudaStreamSynchronize(h->stream));
@@ -1207,14 +1217,15 @@ rlbm_status retile(rlbm_t *h, int P, int kind)
     h->G = h->Gs * (h->N + 1);
     h->plain = kind == kKindPlain || (kind == 0 && prefer_plain(h));
     h->no_tma = kind != 1;
-    h->use_pair = (kind == 2 || kind == 3 || kind == 4) && pair_possible(h, P);
+    h->use_pair = (kind == 2 || kind == 3 || kind == 4 || (kind == kKindGroups && h->R > 1)) && pair_possible(h, P);
+    h->groups = h->use_pair && kind == kKindGroups;
     h->pair_bulk = h->use_pair && kind == 3 && pair_bulk_possible(h) && h->R == 1;
     rlbm_status st = build_tables(h);
     if (st) return st;
     st = setup_tma(h);
     if (st) return st;
     setup_split(h);
-    if (h->use_pair && h->R > 1 && !h->d_split) h->use_pair = false; // no memory for it: the per-tile kernel
+    if (h->use_pair && h->R > 1 && !h->d_split) h->groups = true; // also without memory for the two-pass kernel's ring
     h->use_pair_tma = false;
     if (h->use_pair && kind == 4) {
         st = setup_pair_tma(h);
@@ -1231,10 +1242,11 @@ int kernel_kind(const rlbm_t *h)
     return h->use_tma ? 1 : 0;
 }
 
-// The same, kind 0 with a stand-in told apart.
+// The same, kind 0 with a stand-in and kind 2 with groups told apart.
 int tuned_kind(const rlbm_t *h)
 {
     const int kind = kernel_kind(h);
+    if (kind == 2 && h->groups) return kKindGroups;
     return kind == 0 && stand_in_possible(h) ? (h->plain ? kKindPlain : kKindStandIn) : kind;
 }
 
@@ -1711,7 +1723,7 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
         if (!group_tiling(h->N, h->K, P, gs, ng)) continue;
         if (h->q.onlat && P != 12) continue; // the on-lattice kernel is built for P = 12
         if (P > 2 * h->K) continue;
-        for (int kind : {4, 3, 2, 1, kKindStandIn, kKindPlain, 0}) {
+        for (int kind : {4, 3, 2, kKindGroups, 1, kKindStandIn, kKindPlain, 0}) {
             st = retile(h, P, kind);
             if (st) break;
             if (tuned_kind(h) != kind) continue; // kernel kind not possible for this tiling

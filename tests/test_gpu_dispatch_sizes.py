@@ -65,6 +65,7 @@ def test_two_passes_or_one(nx, ny, K, P, precision):
 
 
 @pytest.mark.parametrize("nx,ny,N,K,precision", [(33, 33, 2, 60, "fp64"), (64, 64, 3, 16, "fp32"), (65, 33, 2, 68, "fp32"),
-                                                 (66, 40, 3, 288, "fp32"), (33, 33, 2, 16, "fp16n")])
+                                                 (66, 40, 3, 288, "fp32"), (33, 33, 2, 16, "fp16n"),
+                                                (8192, 1, 2, 600, "fp32"), (128, 128, 2, 400, "fp32")])
 def test_tuned_choice(nx, ny, N, K, precision):
     run(nx, ny, N, K, precision, None)

@@ -144,8 +144,10 @@ int rlbm_is_onlattice(const rlbm_t *h);
  * from n; rlbm_moments reports this T.  A Bose-Einstein state beyond
  * condensation (no z < 1) is RLBM_ERR_UNPHYSICAL, as a failed Landau frame.
  * Needs g > 0 (RLBM_ERR_ARG); FP64 or FP32 storage, N = 2 or 3 and the
- * off-lattice rule (RLBM_ERR_UNSUPPORTED otherwise).  The per-site part runs in
- * FP64 and the per-tile kernel is used.  Synchronises the stream; the stored
+ * off-lattice rule (RLBM_ERR_UNSUPPORTED otherwise).  FP64 storage: the per-tile
+ * kernel, per-site part in FP64.  FP32 storage: the quadrant kernel where K is a
+ * multiple of P (moments, frame and equilibrium sums in double-float, the (T, z)
+ * solve in FP64), else the per-tile kernel.  Synchronises the stream; the stored
  * populations are kept (call rlbm_init afterwards to start from an equilibrium
  * of the new statistic). */
 rlbm_status rlbm_set_statistics(rlbm_t *h, int statistics, double g);
@@ -194,8 +196,12 @@ rlbm_status rlbm_init_device(rlbm_t *h, const double *d_n, const double *d_T,
  * N^a, T^ab of the streamed populations (Eq. discrete_sum_moments), the
  * Landau frame eps U^a = T^ab U_b with n = U_a N^a and T = eps/(2n), the
  * truncated equilibrium, and relaxation f <- f* - (p.U / p^0 tau)(f* - f^eq)
- * (Eq. discrete-rbe), fused in one kernel per step (one read and one write
- * of every population).  Steps are replayed from a captured CUDA graph. */
+ * (Eq. discrete-rbe), fused in one kernel per step (one read and one write of
+ * every population; two reads in the two-pass kernel of many angles).  Steps are
+ * replayed from a captured CUDA graph, 32 at a time.  Free streaming (tau = inf) of
+ * at most four rows in FP64 or FP32 storage runs up to 32 steps per launch; under
+ * stream capture its launches change buffers as often as the steps would, so that
+ * an even number of captured steps can be replayed. */
 rlbm_status rlbm_step(rlbm_t *h, int nsteps);
 
 /* Landau-frame fields of the stored populations (no streaming): n, eps, T,
@@ -242,7 +248,8 @@ long long rlbm_kernel_launches(const rlbm_t *h);
  * 0 = per-tile kernel; where N <= 3, the collision is finite and K is a
  * multiple of 4, kind 0 also stands for the quadrant kernels for any nx (K a
  * multiple of P in the same list) and, like kind 2, for the two-pass kernel of
- * many angles (bounded waits on its own counters). */
+ * many angles (bounded waits on its own counters); on small grids it stays the
+ * per-tile kernel where that is the faster one. */
 int rlbm_step_kernel_variant(const rlbm_t *h);
 
 /* Select the tiling and step kernel directly (no counterpart in the paper:
@@ -267,8 +274,8 @@ int rlbm_tile_populations(const rlbm_t *h);
  * but the last group are parked in the output buffer between the two passes
  * (FP32 and FP64 storage; rlbm_create refuses such K in 16-bit storage).
  * FP32 storage with N <= 3 and K a multiple of 4 runs such K in the two-pass
- * kernel instead (kind 0, and kind 2 for K a multiple of P), whatever the
- * tiling.  -1 for a NULL handle. */
+ * kernel instead (kind 0, and kind 2 for K a multiple of P), unless the autotuner
+ * finds the groups faster.  -1 for a NULL handle. */
 int rlbm_population_groups(const rlbm_t *h);
 
 /* Autotuner: time every compiled tiling of the step kernel (P populations per

@@ -7,9 +7,6 @@
 
 namespace rlbmk {
 
-// MODE_STEP_LATTICE: a step of the on-lattice rule (perfect streaming by the
-// integer stencil vector of each population, no interpolation).
-// MODE_Q (a bit added to STEP, INIT, MOMENTS): the quantum statistics.
 // How the two sites of a lane of the quadrant kernel lie (rlbm_quad.cuh).
 //   kMapRow     x, x + 1 of one row (nx even): 64 x 1 tiles, 8-byte (4-byte) centre loads
 //   kMapCol     x of rows y, y + 1 (ny > 1, any nx): 32 x 2 tiles; a population needs three
@@ -19,6 +16,9 @@ namespace rlbmk {
 //   kMapSplit   x, x + 32 of one row (ny = 1, any nx): 64 x 1 tiles
 enum QuadMap { kMapRow = 0, kMapCol = 1, kMapSplit = 2 };
 
+// MODE_STEP_LATTICE: a step of the on-lattice rule (perfect streaming by the
+// integer stencil vector of each population, no interpolation).
+// MODE_Q (a bit added to STEP, INIT, MOMENTS): the quantum statistics.
 enum Mode { MODE_STEP = 0, MODE_INIT = 1, MODE_MOMENTS = 2, MODE_STEP_LATTICE = 3, MODE_Q = 4 };
 
 constexpr int kMaxN = 5;

@@ -217,15 +217,17 @@ bool make_onlattice_quadrature(Quad &q)
 
 // FP64 per-site tables (moment folds, projection weights) for the kernels of
 // non-FP64 storage whose per-site part runs in FP64: the init and moments
-// passes, the TMA-staged per-tile kernel, N >= 4 and the quantum statistics.
-// (FP32-storage steps with N <= 3 in the per-tile, batched and
-// two-sites-per-lane kernels run it in double-float from the split tables.)
+// passes, the TMA-staged per-tile kernel, N >= 4 and the quantum statistics of
+// the per-tile kernel.  (FP32-storage steps with N <= 3 in the per-tile, batched,
+// two-sites-per-lane and quadrant kernels run it in double-float from the split
+// tables; the quantum statistics of the quadrant kernel too, but for their (T, z)
+// solve, which is FP64.)
 //  - FP32 storage: an FP32 per-site part carries the conserved moments to a
 //    relative bias of about 4e-7 per step, which the collision accumulates
 //    linearly (1e-5 after a few hundred steps at tau ~ 4);
 //  - N >= 4: the radial projection weights (inverse of a factorial Gram
 //    matrix) cancel too many digits for FP32;
-//  - the quantum statistics: the (T, z) solve.
+//  - the quantum statistics: the (T, z) solve, in the per-tile kernel with all that feeds it.
 // 16-bit storage accumulates in FP32 and solves the Landau frame in
 // double-float (site_landau): its error is set by the storage rounding.
 bool site_fp64_for(int prec, int N, int stat)
@@ -637,7 +639,7 @@ cudaError_t launch(rlbm_t *h, int mode, const rlbmk::KernelArgs &a)
     const bool two_d = h->grid.ny > 1;
     const bool full = h->K == h->R * h->Gs * h->P;
     cudaError_t e;
-    if (h->stat) { // quantum statistics (FP64 per-site part; rlbm_set_statistics checks the rest)
+    if (h->stat) { // quantum statistics, FP64 per-site part (the quadrant kernel's steps do not come here)
         e = h->prec == RLBM_FP64
                 ? rlbmk::launch_quant_f64(mode, h->N, h->P, two_d, full, grid, block, smem, h->stream, a)
                 : rlbmk::launch_quant_f32(mode, h->N, h->P, two_d, full, grid, block, smem, h->stream, a);
@@ -1430,7 +1432,7 @@ rlbm_status rlbm_set_statistics(rlbm_t *h, int statistics, double g)
         RLBM_CUDA(h, cudaMalloc(&h->d_qeta, bytes));
         RLBM_CUDA(h, cudaMemsetAsync(h->d_qeta, 0xff, bytes, h->stream));
     }
-    // the quantum per-site part runs in FP64 (FP32 storage: FP64 site tables)
+    // the per-tile kernel's quantum per-site part runs in FP64 (FP32 storage: FP64 site tables)
     h->site_fp64 = site_fp64_for(h->prec, h->N, statistics);
     return retile(h, h->P, 0);
 }

@@ -1,8 +1,8 @@
 // Tile-staged form of the two-sites-per-lane step (arXiv 2011.06856, Sec. 2.2).
 //
-// The arithmetic is that of rlbm_pair_kernel (two sites per lane as packed
-// f32x2 pairs, the per-site part once per site in two warps); what changes is
-// how the populations reach the registers.  A CTA owns one 64-site tile.  At
+// The arithmetic is that of rlbm_quad_kernel (populations in quadruples of
+// directions, two sites per lane as packed f32x2 pairs, the per-site part in steps
+// shared by the warps); what changes is how the populations reach the registers.  A CTA owns one 64-site tile.  At
 // its start the lanes of warp 0 issue the TMA loads of the whole tile into
 // shared memory -- cp.async.bulk.tensor over the 3D map {nx, ny, npop}:
 //   centre rows  row y of every population, x0 - HX .. x0 + 64 + HX
@@ -14,20 +14,20 @@
 //                give the pull row the weight 0 and join either side), so one
 //                box fetches the right row for a whole chunk;
 // and one mbarrier counts the bytes.  While the copies fly, every thread
-// copies the per-population pair table into shared memory.  After a bounded
+// copies the quad table into shared memory.  After a bounded
 // wait the first pass reads shared memory only, with compile-time offsets; on
 // the domain edges the halo cells outside the grid (zero-filled by the TMA)
 // are first rewritten with their periodic / copy-out source values.  Several
 // CTAs per SM overlap one another's loads, per-site solve and stores.
 //
 // Stores round stochastically: 16-bit ones with the cvt.rs instruction, FP32
-// ones from the FMA residual (relax_pair_sr); random bits from a per-thread
-// LCG (the high halves of its draws, next_bits2).
+// ones from the FMA residual (quad_relax_sr); random bits from QuadBits
+// (rlbm_bits.cuh).
 //
-// One tile per CTA, three CTAs per SM (64 registers, about 71 KB of shared
-// memory with 144 populations in FP16) measured faster than persistent CTAs
-// cycling their tiles through one or two stages: 1.44 ms against 1.61 ms (one
-// stage, three CTAs) and 1.89 ms (two stages, two CTAs) per 2048^2 FP16 step.
+// One tile per CTA measured faster than persistent CTAs cycling their tiles
+// through one or two stages (every population on its own, three CTAs per SM: 1.44 ms
+// against 1.61 ms with one stage and 1.89 ms with two per 2048^2 FP16 step; with four CTAs
+// per SM 1.27, with quadruples of directions 0.90).
 //
 // Every wait is bounded: on expiry the CTA sets bit 1 of the status word,
 // waits (again bounded) for its copies and returns without storing.

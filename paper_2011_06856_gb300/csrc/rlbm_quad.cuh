@@ -18,7 +18,7 @@
 //  - needs one table entry per quad: (c,c,s,s), (cos 2t, cos 2t, sin 2t, sin 2t) and
 //    for N = 3 the third harmonic.
 // The weights w_i of a shell are equal, so they are folded into its projection weights
-// (KernelArgs::rq, rq2).
+// (KernelArgs::rq).
 //
 // The per-site part uses closed forms: the moments of the boosted rest-frame direction
 // q on the light cone are

@@ -27,7 +27,7 @@
 // One tile per CTA measured faster than persistent CTAs cycling their tiles
 // through one or two stages (every population on its own, three CTAs per SM: 1.44 ms
 // against 1.61 ms with one stage and 1.89 ms with two per 2048^2 FP16 step; with four CTAs
-// per SM 1.27, with quadruples of directions 0.90).
+// per SM 1.27, with quadruples of directions 0.91).
 //
 // Every wait is bounded: on expiry the CTA sets bit 1 of the status word,
 // waits (again bounded) for its copies and returns without storing.

@@ -12,7 +12,7 @@
 // leaves the shells' coefficients in a ring in global memory; a pass B CTA streams the
 // same quads again, lag tiles later, and relaxes them.  Nobody waits and any CTA can run
 // next to any other: 490 us (2.45 instructions a cycle and SM against 1.5), 1000^2 9.8 to
-// 7.3 ms.  The price is the second read and pull, about a third of the arithmetic; it
+// 7.3 ms; with the residual of the FP32 stores 505 us and 7.6 ms.  The price is the second read and pull, about a third of the arithmetic; it
 // comes from the L2 while lag tiles fit there (K up to about 250).
 //
 // CTAs are small (four warps, five per SM, 96 registers): a CTA's start and end (ticket,

@@ -113,7 +113,7 @@ def measured_peaks():
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
     for f in ("rlbm_device.cuh", "rlbm_launch.cuh", "rlbm_args.h", "rlbm_pair.cuh", "rlbm_df64.cuh",
-              "rlbm_pair_tma.cuh", "rlbm_tma.cuh", "rlbm_quad.cuh", "rlbm_quad64.cuh", "rlbm_quad_split.cuh"):
+              "rlbm_pair_tma.cuh", "rlbm_tma.cuh", "rlbm_bits.cuh", "rlbm_quad.cuh", "rlbm_quad64.cuh", "rlbm_quad_split.cuh"):
         with open(os.path.join(ROOT, "paper_2011_06856_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -397,7 +397,7 @@ def run_batch(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_source": src, "traffic": None,
                          "kernel": "rlbm_batch_kernel" if mode_used == "persistent"
-                         else "per-problem step kernels (rlbm_pair_kernel / rlbm_kernel)"},
+                         else "per-problem step kernels (rlbm_quad_kernel / rlbm_kernel)"},
             "cpu_baseline": None,
             "e2e": None, "gpu_launches": int(launches), "clocks": clocks}
     if rank == 0:
@@ -634,19 +634,29 @@ def main():
                 sim.autotune(8)
     tiling = {"populations_per_warp": sims[0].tile_populations, "kernel": sims[0].step_kernel,
               "population_groups_per_warp": sims[0].population_groups}
-    kernel_names = {"per-tile": "rlbm_kernel<MODE_STEP>", "tma": "rlbm_step_tma",
-                    "pair": "rlbm_pair_kernel", "pair-bulk": "rlbm_pair_kernel (bulk-staged)",
+    kernel_names = {"tma": "rlbm_step_tma", "pair-bulk": "rlbm_pair_kernel (bulk-staged)",
                     "pair-tma": "rlbm_pair_tma_kernel"}
 
     def kernel_name(sim):
-        if sim.statistics != "mj":
-            return "rlbm_kernel<MODE_STEP | MODE_Q>"
+        """The step kernel of the handle's kind and tiling (include/rlbm.h,
+        rlbm_step_kernel_variant); kinds 0 and 2 stand for several."""
         if sim.onlattice:
             return "rlbm_kernel<MODE_STEP_LATTICE>"
-        if sim.population_groups > 1:
-            return {"pair": "rlbm_pair_groups_kernel",
-                    "per-tile": "rlbm_kernel<MODE_STEP> (population groups)"}[sim.step_kernel]
-        return kernel_names[sim.step_kernel]
+        if sim.step_kernel in kernel_names:
+            return kernel_names[sim.step_kernel]
+        P, fp64 = sim.tile_populations, sim.precision == "fp64"
+        if math.isinf(sim.tau) and sim.ny <= 4 and sim.precision in ("fp64", "fp32"):
+            return "rlbm_free_kernel"
+        if sim.step_kernel == "pair" and sim.population_groups > 1:
+            return "rlbm_quad_split_kernel or rlbm_pair_groups_kernel"
+        quad = (math.isfinite(sim.tau) and sim.N <= 3 and P in (8, 12, 16, 24, 32) and sim.K % P == 0
+                and sim.population_groups == 1)
+        if sim.statistics != "mj":
+            return "rlbm_quad_kernel" if quad and not fp64 else "rlbm_kernel<MODE_STEP | MODE_Q>"
+        if quad:
+            return "rlbm_quad64_kernel" if fp64 else "rlbm_quad_kernel"
+        many = math.isfinite(sim.tau) and sim.N <= 3 and sim.K % 4 == 0 and sim.K >= 64 and not fp64
+        return "rlbm_quad_split_kernel (rlbm_kernel<MODE_STEP> on a small grid)" if many else "rlbm_kernel<MODE_STEP>"
 
     # the step launches are timed inside the timed region, on the streams they
     # are issued on: events before and after every problem's run of steps; the

@@ -1719,6 +1719,9 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
     RLBM_CUDA(h, cudaEventCreate(&e1));
     TuneChoice best{h->P, tuned_kind(h), 1e30f};
     const long long launches0 = h->launches;
+    // From 65536 sites on (256^2) the quadrant and two-pass kernels were faster than the per-tile
+    // and groups kernels on every tiling measured: no trials of those there.
+    const bool small = (long long)h->grid.nx * h->grid.ny < 65536;
     rlbm_status st = RLBM_OK;
     for (int P : sizes) {
         int gs = 0, ng = 0;
@@ -1726,6 +1729,7 @@ rlbm_status rlbm_autotune(rlbm_t *h, int launches_per_trial, float *best_ms)
         if (h->q.onlat && P != 12) continue; // the on-lattice kernel is built for P = 12
         if (P > 2 * h->K) continue;
         for (int kind : {4, 3, 2, kKindGroups, 1, kKindStandIn, kKindPlain, 0}) {
+            if (!small && (kind == kKindGroups || kind == kKindPlain)) continue;
             st = retile(h, P, kind);
             if (st) break;
             if (tuned_kind(h) != kind) continue; // kernel kind not possible for this tiling
